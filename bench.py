@@ -353,7 +353,7 @@ def graph_comparison(A, stream, precision, nsteps=200):
 def uniform_roofline(A, stream, precision, J=5, nsteps=5):
     """The fused stage kernel on a uniform periodic grid (unit cube at level J: 8^J blocks of
     17^3, Taylor-Green, the config-1 physics): its CUDA-event time per launch over nsteps RK4
-    steps and the algorithmic bandwidth (64 words per point and RK4 step without a mask)."""
+    steps and the algorithmic bandwidth (52 words per point and RK4 step without a mask)."""
     import torch
     nb = 8 ** J
     grid = dict(nroot=(1, 1, 1), root_len=1.0, Bs=17, g=4, Jmin=J, Jmax=J, precision=precision, max_blocks=nb,
@@ -577,7 +577,7 @@ def fullscale_plate(A, stream, Bs=33, Jmax=7, max_blocks=29000, nsteps=20, adj_B
     del f
     torch.cuda.empty_cache()
     out = {"workload": f"flapping plate in the box 8^3, Bs = {Bs}, levels 2..{Jmax}, FP32, {nsteps} adaptive steps",
-           # the events around each stage also hold the plate's solid-velocity source kernel
+           # the plate's solid-velocity source is part of the stage kernel
            "autotune": {"stage_variant": tuning["stage_variant"], "stage_ms": tuning["stage_ms"]},
            "stage_kernel": {"ms_per_launch_with_solid_source": st["stage_ms"] / 4,
                             "achieved_gbs": stage_gbs, "frac": stage_gbs / peak if stage_gbs else None,
@@ -976,9 +976,7 @@ def main():
                          "frac": round(stage_bytes / ((stage_ms + sync_ms) * 1e-3) / 1e9 / peak, 4),
                          "sync_ms_per_stage": sync_ms / launches_stage,
                          "stage_ms_per_stage": stage_ms / launches_stage}}
-        roof["kernel"] = {0: "k_stage_pair<17> (fused RHS + RK4 stage, 2 points per thread)",
-                          1: "k_stage<float,17> (fused RHS + RK4 stage)",
-                          2: "k_stage<float,17,TMA> (fused RHS + RK4 stage, bulk-copy staging)"}[tuning["stage_variant"]]
+        roof["kernel"] = "k_stage<float,17> (fused RHS + RK4 stage)"
 
         # end to end through the C-ABI with host buffers: write state, step, read state
         e2e = None
@@ -1095,12 +1093,8 @@ def main():
             "adjoint": adjoint,
             "uniform_roofline": uniform,
             "autotune": {"fine_wins_ctas_per_sm": tuned[0], "slab_ctas_per_sm": tuned[1],
-                         "stage_kernel": {0: "pair (2 points/thread, packed f32x2)",
-                                          1: "point (1 point/thread)",
-                                          2: "point, bulk-copy (TMA) staging of U/acc/chi",
-                                          3: "point, a block's rows over two CTAs"}[tuning["stage_variant"]],
-                         "stage2_ms": {"pair": tuning["stage_ms"][0], "point": tuning["stage_ms"][1],
-                                       "point_tma": tuning["stage_ms"][2], "point_rows": tuning["stage_ms"][3]}},
+                         "stage_kernel": "point (1 point/thread)",
+                         "stage2_ms": tuning["stage_ms"][1]},
             "clocks": clk,
         }
         print(json.dumps(line), flush=True)

@@ -246,37 +246,30 @@ acm_status acm_rk4_steps_batch(acm_forest* const* forests, int n, int nsteps, do
 /* Autotuner: on the current grid, time the two task-list kernels of the per-stage ghost
  * synchronisation -- fine wins and the coarse-face halo slabs -- for each number of CTAs per SM
  * walking the list (fine wins 2, 4, 8, 16; slabs 1, 2, 3) and keep the fastest of each for this
- * forest (either output may be NULL).  FP32 forests also time the forms of the fused stage
- * kernel (ACM_STAGE_* below; blocks of 33^3 have one) on one RK stage of the live grid and keep
- * the fastest.  Like every synchronisation it first lets finer leaves' values win on shared
+ * forest (either output may be NULL).  FP32 forests also time one launch of the fused stage
+ * kernel on the live grid.  Like every synchronisation it first lets finer leaves' values win on shared
  * boundary points of U; nothing else of the state changes (the stage timing writes only the
  * accumulator and a stage register, which every step rewrites before reading).  Synchronises
  * the stream.  No counterpart in the paper. */
 acm_status acm_autotune(acm_forest* f, int* fw_ctas, int* slab_ctas);
 
-/* Forms of the fused right-hand side + RK4 stage kernel (Sec. 2.1-2.3): ACM_STAGE_POINT, one
- * point per thread (the default); ACM_STAGE_PAIR, two x-adjacent points per thread with packed
- * FP32x2 arithmetic (FP32 forests only: fewer instructions, half the resident threads);
- * ACM_STAGE_POINT_TMA, one point per thread with the planes of U, the RK accumulator and the mask
- * brought into a shared-memory ring by mbarrier-tracked bulk copies one plane ahead (FP32 forests
- * only); ACM_STAGE_POINT_ROWS, one point per thread with a block's rows split over CTAs of 9 rows (FP32,
- * Bs = 17: two CTAs of 9 and 8 rows; Bs = 33: four of 9, 9, 9 and 6 rows; smaller CTAs, more of
- * them per SM, each reading the rows next to its own like a halo).  All compute every point by
- * the same formula; ACM_STAGE_POINT, ACM_STAGE_POINT_TMA and ACM_STAGE_POINT_ROWS give bitwise
- * equal results, ACM_STAGE_PAIR differs in FP32 rounding order.  FP64 forests always use
- * ACM_STAGE_POINT; forests of 33^3 blocks use ACM_STAGE_POINT_ROWS or else their three-CTA
- * form (11 rows each) for ACM_STAGE_POINT, ACM_STAGE_PAIR and ACM_STAGE_POINT_TMA. */
+/* Names of the forms that the fused right-hand side + RK4 stage kernel (Sec. 2.1-2.3) has had:
+ * ACM_STAGE_POINT, one point per thread; ACM_STAGE_PAIR, two x-adjacent points per thread;
+ * ACM_STAGE_POINT_TMA, one point per thread with its planes staged by bulk copies;
+ * ACM_STAGE_POINT_ROWS, a block's rows split over CTAs.  There is one kernel now, which does all of
+ * this for the size at hand (bulk-staged planes, packed FP32x2 arithmetic, 33^3 blocks split by
+ * rows): every name selects it, and the results do not depend on the name. */
 #define ACM_STAGE_PAIR 0
 #define ACM_STAGE_POINT 1
 #define ACM_STAGE_POINT_TMA 2
 #define ACM_STAGE_POINT_ROWS 3
-/* Force the stage kernel's form (until the next acm_autotune); drops a captured graph.
- * ACM_EINVAL for another value. */
+/* Accepts the names above (they select the same kernel); drops a captured graph.  ACM_EINVAL for
+ * another value. */
 acm_status acm_set_stage_variant(acm_forest* f, int variant);
 
 /* The launch knobs in use: CTAs per SM of the fine-wins and slab kernels, the stage kernel's
- * form, and the autotuner's median times (ms) of one stage launch in each form (indexed by
- * ACM_STAGE_*; 0 until it has timed them). */
+ * form (ACM_STAGE_POINT), and in stage_ms[ACM_STAGE_POINT] the autotuner's median time (ms) of one
+ * stage launch of an FP32 forest (0 until it has timed it; the other entries stay 0). */
 typedef struct {
   int fw_ctas_per_sm, slab_ctas_per_sm, stage_variant;
   float stage_ms[4];
@@ -441,7 +434,7 @@ acm_status acm_read_mask(acm_forest* f, void* out, int64_t n_elems, int on_devic
 /* Per-kernel timing of the last acm_rk4_step with timing enabled (CUDA events recorded on the
  * forest's stream around each stage's synchronisation kernels and fused stage kernel; read
  * when this is called, which waits for the last of them), milliseconds summed over the four
- * stages, and the algorithmic bytes of the four fused stage kernels (per point 64 words of
+ * stages, and the algorithmic bytes of the four fused stage kernels (per point 52 words of
  * register traffic, plus 4 words of mask when a mask is set). */
 typedef struct {
   double stage_ms;        /* fused RHS+RK4 stage kernels                                    */

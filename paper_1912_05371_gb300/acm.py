@@ -306,10 +306,8 @@ class Forest:
         return a.value, b.value
 
     def set_stage_variant(self, variant):
-        """Force the stage kernel's form: ACM_STAGE_POINT (one point per thread), ACM_STAGE_PAIR
-        (two points per thread, FP32), ACM_STAGE_POINT_TMA (one point per thread, bulk-copy
-        staging, FP32) or ACM_STAGE_POINT_ROWS (one point per thread, a 17^3 block's rows over
-        two CTAs, FP32)."""
+        """Accepts ACM_STAGE_POINT, ACM_STAGE_PAIR, ACM_STAGE_POINT_TMA and ACM_STAGE_POINT_ROWS: one
+        stage kernel serves them all, with the same results."""
         self._check(self.L.acm_set_stage_variant(self.h, int(variant)))
 
     def tuning(self):

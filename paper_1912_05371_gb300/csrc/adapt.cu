@@ -6,6 +6,7 @@
 // restrict or predict, then copy), Sec. 2.2 (smoothed mask, force by midpoint rule).
 #include <algorithm>
 #include <atomic>
+#include <type_traits>
 
 #include "common.cuh"
 #include "kernels.hpp"
@@ -53,7 +54,8 @@ __device__ __forceinline__ void gather(T* dst, int n, F&& val) {
 // task = (rank, box index d of a REFINED neighbour box).  Points of the block's boundary lying
 // in box d: coordinate 0 / M where d is -1 / +1, the whole range where d is 0.  The CTAs walk
 // the task list (its length is on the device).
-template <typename T, int BS>
+// PM: the register is point-major (a point's components side by side).
+template <typename T, int BS, bool PM>
 __device__ __forceinline__ void fine_wins_task(T* reg, const int2 tk, const int32_t* nbh_all, const int32_t* blist) {
   using L = Lay<T, BS>;
   constexpr int M = L::M;
@@ -80,18 +82,24 @@ __device__ __forceinline__ void fine_wins_task(T* reg, const int2 tk, const int3
     }
     const int s = nbh[8 * d + c];
     if (s < 0) continue;
+    if (PM) {
+      struct alignas(16) Q { T v[4]; };
+      *reinterpret_cast<Q*>(reg + (size_t)me * L::BLK + 4 * ((p[2] * BS + p[1]) * BS + p[0])) =
+          *reinterpret_cast<const Q*>(reg + (size_t)s * L::BLK + 4 * ((l[2] * BS + l[1]) * BS + l[0]));
+    } else {
 #pragma unroll
-    for (int f = 0; f < 4; ++f)
-      reg[(size_t)me * L::BLK + (size_t)f * L::FS + L::idx(p[0], p[1], p[2])] =
-          reg[(size_t)s * L::BLK + (size_t)f * L::FS + L::idx(l[0], l[1], l[2])];
+      for (int f = 0; f < 4; ++f)
+        reg[(size_t)me * L::BLK + (size_t)f * L::FS + L::idx(p[0], p[1], p[2])] =
+            reg[(size_t)s * L::BLK + (size_t)f * L::FS + L::idx(l[0], l[1], l[2])];
+    }
   }
 }
 
-template <typename T, int BS>
+template <typename T, int BS, bool PM>
 __global__ void __launch_bounds__(kNT) k_fine_wins(T* reg, const int2* tasks, const int32_t* ntasks,
                                                     const int32_t* nbh_all, const int32_t* blist) {
   const int nt = *ntasks;
-  for (int t = blockIdx.x; t < nt; t += gridDim.x) fine_wins_task<T, BS>(reg, tasks[t], nbh_all, blist);
+  for (int t = blockIdx.x; t < nt; t += gridDim.x) fine_wins_task<T, BS, PM>(reg, tasks[t], nbh_all, blist);
 }
 
 // ---- (2) coarse-face halo slabs ------------------------------------------------------------------
@@ -138,7 +146,18 @@ __device__ __forceinline__ int edge_index(int t0, int t1) {
   return 2 * BS + (BS - 2) + t1 - 1;
 }
 
+// PM: the register and the slabs are point-major.  The cached lookups are component-major offsets in
+// either case (the first stage, which fills the cache, reads U): pm_offset converts them.
 template <typename T, int BS>
+__device__ __forceinline__ long long pm_offset(long long o) {
+  using L = Lay<T, BS>;
+  const unsigned u = (unsigned)o, s = u / (unsigned)L::BLK, r = u % (unsigned)L::BLK;
+  return (long long)s * L::BLK + 4ll * ((r / (unsigned)L::PP) * (BS * BS) + r % (unsigned)L::PP);
+}
+template <typename T>
+struct alignas(16) Quad { T v[4]; };
+
+template <typename T, int BS, bool PM>
 __global__ void __launch_bounds__(SlabSmem<T, BS>::NT, SlabSmem<T, BS>::MINB)
 k_coarse_slabs(const T* reg, T* slab, const int4* tasks, const int32_t* ntasks, const int32_t* nbh_all, uint32_t* offc,
                int use_cache) {
@@ -170,6 +189,18 @@ k_coarse_slabs(const T* reg, T* slab, const int4* tasks, const int32_t* ntasks, 
     else if (ax == 1) { *x = t0; *y = nl; *z = t1; }
     else { *x = t0; *y = t1; *z = nl; }
   };
+  // the four components at a (component-major) offset, or `none` where there is none
+  auto load_four = [&](long long o, T none, T (&v)[4]) {
+    if (PM) {
+      Quad<T> q{{none, none, none, none}};
+      if (o >= 0) q = *reinterpret_cast<const Quad<T>*>(reg + pm_offset<T, BS>(o));
+#pragma unroll
+      for (int f = 0; f < 4; ++f) v[f] = q.v[f];
+    } else {
+#pragma unroll
+      for (int f = 0; f < 4; ++f) v[f] = o >= 0 ? reg[o + (long long)f * L::FS] : none;
+    }
+  };
   // leaf lookups of the halo column (t0, t1) on the face's boundary lines (component 0
   // offsets; component f is FS further), and its values
   auto edge_values = [&](int t0, int t1, long long (&eo)[3], T (&ev)[3][4]) {
@@ -190,9 +221,7 @@ k_coarse_slabs(const T* reg, T* slab, const int4* tasks, const int32_t* ntasks, 
       }
     }
 #pragma unroll
-    for (int l = 0; l < 3; ++l)
-#pragma unroll
-      for (int f = 0; f < 4; ++f) ev[l][f] = eo[l] >= 0 ? reg[eo[l] + (long long)f * L::FS] : T(0);
+    for (int l = 0; l < 3; ++l) load_four(eo[l], T(0), ev[l]);
   };
   // with one column per thread its edge values are loaded with the patch, before the passes
   const bool col = tid < BS * BS;
@@ -220,10 +249,7 @@ k_coarse_slabs(const T* reg, T* slab, const int4* tasks, const int32_t* ntasks, 
   }
   T pv[U][4];
 #pragma unroll
-  for (int k = 0; k < U; ++k)
-#pragma unroll
-    for (int f = 0; f < 4; ++f)
-      pv[k][f] = off[k] >= 0 ? reg[off[k] + (long long)f * L::FS] : T(__longlong_as_double(0x7ff8000000000000ll));
+  for (int k = 0; k < U; ++k) load_four(off[k], T(__longlong_as_double(0x7ff8000000000000ll)), pv[k]);
 #pragma unroll
   for (int k = 0; k < U; ++k)
     if (off[k] != -2)
@@ -249,6 +275,7 @@ k_coarse_slabs(const T* reg, T* slab, const int4* tasks, const int32_t* ntasks, 
   __syncthreads();
   // across the face: column (t0, t1)
   auto column_out = [&](int t0, int t1, const long long (&eo)[3], const T (&ev)[3][4]) {
+    Quad<T> q[3];                                   // [layer]: the column's values, point-major
     const T w[4] = {T(-1) / T(16), T(9) / T(16), T(9) / T(16), T(-1) / T(16)};
 #pragma unroll
     for (int f = 0; f < 4; ++f) {
@@ -271,8 +298,14 @@ k_coarse_slabs(const T* reg, T* slab, const int4* tasks, const int32_t* ntasks, 
             v = cn[c >> 1];
           }
         }
-        slab[((((size_t)tk.z * 4 + f) * 3 + (l - 1)) * BS + t1) * BS + t0] = v;
+        if (PM) q[l - 1].v[f] = v;
+        else slab[((((size_t)tk.z * 4 + f) * 3 + (l - 1)) * BS + t1) * BS + t0] = v;
       }
+    }
+    if (PM) {
+#pragma unroll
+      for (int l = 0; l < 3; ++l)
+        *reinterpret_cast<Quad<T>*>(slab + ((((size_t)tk.z * 3 + l) * BS + t1) * BS + t0) * 4) = q[l];
     }
   };
   if (S::ONE) {
@@ -1485,38 +1518,6 @@ __global__ void __launch_bounds__(ColCfg<BS>::NT) k_mask(T* chi, const int32_t* 
 }
 
 // ---- (9) diagnostics: raw per-block sums over the half-open points [0, M-1]^3 -----------------
-// Penalization source of a rotating rigid body (mask kind 2): S = chi (omega x (x - x_0)) / C_eta,
-// added to the stage outputs (out += c_out S, acc += c_acc S).  FP64 arithmetic per point is
-// avoided for FP32 fields: the pose arrives in double and is converted once.
-template <typename T, int BS>
-__global__ void __launch_bounds__(kNT) k_solid_source(T* out, T* acc, const T* chi, const int32_t* blist,
-                                                      const int4* binfo, const PhysK ph, const MaskK m, double c_out,
-                                                      double c_acc, int acc_too) {
-  using L = Lay<T, BS>;
-  constexpr int M = L::M;
-  const int slot = blist[blockIdx.x];
-  const int4 bi = binfo[blockIdx.x];
-  const T hT = T(ph.h[bi.x]);
-  const T w0 = T(m.p[19]), w1 = T(m.p[20]), w2 = T(m.p[21]);
-  const T x0 = T(m.p[9]), y0 = T(m.p[10]), z0 = T(m.p[11]);
-  const T ci = T(ph.inv_ceta), co = T(c_out), ca = T(c_acc);
-  const size_t base = (size_t)slot * L::BLK;
-  for (int t = threadIdx.x; t < BS * BS * BS; t += kNT) {
-    const int x = t % BS, y = (t / BS) % BS, z = t / (BS * BS);
-    const int pi = L::idx(x, y, z);
-    const T c = chi[(size_t)slot * L::FS + pi];
-    if (c == T(0)) continue;
-    const T rx = T(lattice(ph, bi, 0, x, M)) * hT - x0;
-    const T ry = T(lattice(ph, bi, 1, y, M)) * hT - y0;
-    const T rz = T(lattice(ph, bi, 2, z, M)) * hT - z0;
-    const T s[3] = {c * ci * (w1 * rz - w2 * ry), c * ci * (w2 * rx - w0 * rz), c * ci * (w0 * ry - w1 * rx)};
-    for (int a = 0; a < 3; ++a) {
-      out[base + (size_t)a * L::FS + pi] += co * s[a];
-      if (acc_too) acc[base + (size_t)a * L::FS + pi] += ca * s[a];
-    }
-  }
-}
-
 // Per block sums over the half-open points of chi u_s (force of a moving body, Sec. 2.2).
 template <typename T, int BS>
 __global__ void __launch_bounds__(kNT) k_solid_moment(const T* chi, const int32_t* blist, const int4* binfo,
@@ -1660,34 +1661,51 @@ LayoutInfo layout_info(int precision, int Bs) {
 
 template <typename T>
 void launch_fine_wins(int Bs, T* reg, const int2* tasks, const int32_t* ntasks, int64_t max_tasks,
-                      const int32_t* nbh, const int32_t* blist, int ctas_per_sm, cudaStream_t st) {
+                      const int32_t* nbh, const int32_t* blist, int ctas_per_sm, bool point_major, cudaStream_t st) {
   if (max_tasks <= 0) return;
   const int64_t g = std::min<int64_t>(max_tasks, (int64_t)std::max(1, ctas_per_sm) * sm_count());
-  ACM_BS_DISPATCH(Bs, k_fine_wins, <<<grid1(g), kNT, 0, st>>>(reg, tasks, ntasks, nbh, blist));
+  auto go = [&](auto pm) {
+    constexpr bool PM = decltype(pm)::value;
+    if (Bs == 33) {
+      if constexpr (sizeof(T) == 4) k_fine_wins<T, 33, PM><<<grid1(g), kNT, 0, st>>>(reg, tasks, ntasks, nbh, blist);
+    } else if (Bs == 17) {
+      k_fine_wins<T, 17, PM><<<grid1(g), kNT, 0, st>>>(reg, tasks, ntasks, nbh, blist);
+    } else {
+      k_fine_wins<T, 9, PM><<<grid1(g), kNT, 0, st>>>(reg, tasks, ntasks, nbh, blist);
+    }
+  };
+  if (point_major) go(std::true_type{});
+  else go(std::false_type{});
 }
-template <typename T, int BS>
+template <typename T, int BS, bool PM>
 void launch_coarse_slabs_bs(const T* reg, T* slab, const int4* tasks, const int32_t* ntasks, int64_t max_tasks,
                             const int32_t* nbh, uint32_t* offc, int use_cache, int ctas_per_sm, cudaStream_t st) {
   static std::atomic<unsigned long long> opted{0};   // devices whose context has the opt-in
-  smem_opt_in(k_coarse_slabs<T, BS>, SlabSmem<T, BS>::bytes, opted);
+  smem_opt_in(k_coarse_slabs<T, BS, PM>, SlabSmem<T, BS>::bytes, opted);
   // CTAs walking the task list: ctas_per_sm per SM (at most 3 are resident for Bs = 17)
   const int64_t g = std::min<int64_t>(max_tasks, (int64_t)std::max(1, ctas_per_sm) * sm_count());
-  k_coarse_slabs<T, BS><<<grid1(g), SlabSmem<T, BS>::NT, SlabSmem<T, BS>::bytes, st>>>(reg, slab, tasks, ntasks, nbh,
-                                                                                       offc, use_cache);
+  k_coarse_slabs<T, BS, PM><<<grid1(g), SlabSmem<T, BS>::NT, SlabSmem<T, BS>::bytes, st>>>(reg, slab, tasks, ntasks, nbh,
+                                                                                           offc, use_cache);
 }
 template <typename T>
 void launch_coarse_slabs(int Bs, const T* reg, T* slab, const int4* tasks, const int32_t* ntasks, int64_t max_tasks,
-                         const int32_t* nbh, uint32_t* offc, int use_cache, int ctas_per_sm, cudaStream_t st) {
+                         const int32_t* nbh, uint32_t* offc, int use_cache, int ctas_per_sm, bool point_major,
+                         cudaStream_t st) {
   if (max_tasks <= 0) return;
-  if (Bs == 33) {
-    // one CTA per SM is resident (166 KB of shared memory)
-    if constexpr (sizeof(T) == 4)
-      launch_coarse_slabs_bs<T, 33>(reg, slab, tasks, ntasks, max_tasks, nbh, offc, use_cache, 1, st);
-  } else if (Bs == 17) {
-    launch_coarse_slabs_bs<T, 17>(reg, slab, tasks, ntasks, max_tasks, nbh, offc, use_cache, ctas_per_sm, st);
-  } else {
-    launch_coarse_slabs_bs<T, 9>(reg, slab, tasks, ntasks, max_tasks, nbh, offc, use_cache, ctas_per_sm, st);
-  }
+  auto go = [&](auto pm) {
+    constexpr bool PM = decltype(pm)::value;
+    if (Bs == 33) {
+      // one CTA per SM is resident (166 KB of shared memory)
+      if constexpr (sizeof(T) == 4)
+        launch_coarse_slabs_bs<T, 33, PM>(reg, slab, tasks, ntasks, max_tasks, nbh, offc, use_cache, 1, st);
+    } else if (Bs == 17) {
+      launch_coarse_slabs_bs<T, 17, PM>(reg, slab, tasks, ntasks, max_tasks, nbh, offc, use_cache, ctas_per_sm, st);
+    } else {
+      launch_coarse_slabs_bs<T, 9, PM>(reg, slab, tasks, ntasks, max_tasks, nbh, offc, use_cache, ctas_per_sm, st);
+    }
+  };
+  if (point_major) go(std::true_type{});
+  else go(std::false_type{});
 }
 size_t slab_offset_words(int Bs) {
   return Bs == 33 ? SlabSmem<float, 33>::NOFF : (Bs == 17 ? SlabSmem<float, 17>::NOFF : SlabSmem<float, 9>::NOFF);
@@ -1799,12 +1817,6 @@ void launch_mask(int Bs, T* chi, const int32_t* blist, const int32_t* ranks, int
   }
 }
 template <typename T>
-void launch_solid_source(int Bs, T* out, T* acc, const T* chi, const int32_t* blist, const int4* binfo, int64_t n,
-                         const PhysK& p, const MaskK& m, double c_out, double c_acc, int acc_too, cudaStream_t st) {
-  if (n <= 0) return;
-  ACM_BS_DISPATCH(Bs, k_solid_source, <<<grid1(n), kNT, 0, st>>>(out, acc, chi, blist, binfo, p, m, c_out, c_acc, acc_too));
-}
-template <typename T>
 void launch_solid_moment(int Bs, const T* chi, const int32_t* blist, const int4* binfo, int64_t n, const PhysK& p,
                          const MaskK& m, double* out, cudaStream_t st) {
   if (n <= 0) return;
@@ -1836,8 +1848,8 @@ void launch_scatter(int Bs, const T* dense, T* reg, const int32_t* blist, int64_
 }
 
 #define ACM_INST(T)                                                                                        \
-  template void launch_fine_wins<T>(int, T*, const int2*, const int32_t*, int64_t, const int32_t*, const int32_t*, int, cudaStream_t); \
-  template void launch_coarse_slabs<T>(int, const T*, T*, const int4*, const int32_t*, int64_t, const int32_t*, uint32_t*, int, int, cudaStream_t); \
+  template void launch_fine_wins<T>(int, T*, const int2*, const int32_t*, int64_t, const int32_t*, const int32_t*, int, bool, cudaStream_t); \
+  template void launch_coarse_slabs<T>(int, const T*, T*, const int4*, const int32_t*, int64_t, const int32_t*, uint32_t*, int, int, bool, cudaStream_t); \
   template void launch_sync_ext<T>(int, const T*, T*, int, const int32_t*, int64_t, const int32_t*, int, cudaStream_t); \
   template void launch_details<T>(int, const T*, const T*, const int32_t*, const int32_t*, const int32_t*, int64_t, const unsigned long long*, double*, double*, cudaStream_t); \
   template void launch_maxnorm<T>(int, const T*, const int32_t*, int64_t, unsigned long long*, cudaStream_t); \
@@ -1848,7 +1860,6 @@ void launch_scatter(int Bs, const T* dense, T* reg, const int32_t* blist, int64_
   template void launch_ic<T>(int, T*, const int32_t*, const int32_t*, int64_t, const int4*, const PhysK&, const IcK&, cudaStream_t); \
   template void launch_mask<T>(int, T*, const int32_t*, const int32_t*, int64_t, const int4*, const PhysK&, const MaskK&, cudaStream_t); \
   template void launch_diag<T>(int, const T*, const T*, const int32_t*, int64_t, double*, cudaStream_t);   \
-  template void launch_solid_source<T>(int, T*, T*, const T*, const int32_t*, const int4*, int64_t, const PhysK&, const MaskK&, double, double, int, cudaStream_t); \
   template void launch_solid_moment<T>(int, const T*, const int32_t*, const int4*, int64_t, const PhysK&, const MaskK&, double*, cudaStream_t); \
   template void launch_gather<T>(int, const T*, T*, const int32_t*, int64_t, int, cudaStream_t);          \
   template void launch_scatter<T>(int, const T*, T*, const int32_t*, int64_t, int, cudaStream_t);

@@ -38,6 +38,9 @@ namespace {
 
 constexpr int kNA = 256;
 
+// faces: 0 -x, 1 +x, 2 -y, 3 +y, 4 -z, 5 +z ; box index of the face neighbour
+__constant__ int kFaceBox[6] = {12, 14, 10, 16, 4, 22};
+
 __device__ __forceinline__ double lattice_coord(const PhysK& ph, int4 bi, int a, int i, int M, double h) {
   const int g = a == 0 ? bi.y : (a == 1 ? bi.z : bi.w);
   const long long N = ((long long)ph.nroot[a] << bi.x) * M;
@@ -207,9 +210,8 @@ k_adj_stage(const AdjStageK<T> a, const TopoK tp, const PhysK ph, const MaskK m)
   const int rank = blockIdx.x / C::NS, part = blockIdx.x % C::NS;
   const int slot = tp.blist[rank];
   const int4 bi = tp.binfo[rank];
-  const int* nbh = tp.nbh + (size_t)rank * kNbhStride;
   const int y0 = part * RY, ny = BS - y0 < RY ? BS - y0 : RY;    // this CTA's rows
-  stage_faces(tid, nbh, tp.slabidx, rank, ftype, fs);
+  stage_faces(tid, tp.faces, rank, ftype, fs);
   stage_sponge<T, BS>(tid, ph, bi, sp);
   // the kappa planes' halos stay zero (sources outside the block weigh nothing)
   for (int i = tid; i < 2 * C::NC * PW; i += NT) buf[i] = T(0);

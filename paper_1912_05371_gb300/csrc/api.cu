@@ -52,6 +52,7 @@ struct acm_forest {
   int4* d_binfo = nullptr;
   int32_t* d_blist = nullptr;
   int32_t* d_slabidx = nullptr;
+  int32_t* d_faces = nullptr;
   int2* d_fw = nullptr;
   int4* d_slabt = nullptr;
   int4* d_reft = nullptr;
@@ -87,8 +88,7 @@ struct acm_forest {
   // launch knobs chosen by acm_autotune (defaults until it runs)
   int tune_fw_ctas = 8;            // fine-wins kernel: CTAs per SM walking the task list
   int tune_slab_ctas = 3;          // coarse-face slab kernel: CTAs per SM walking the task list
-  int stage_variant = acm::kStagePoint;  // FP32 stage kernel: one point per thread, or two
-  float tune_stage_ms[4] = {0.f, 0.f, 0.f, 0.f};   // the autotuner's times of the forms (FP32)
+  float tune_stage_ms = 0.f;       // the autotuner's time of one stage launch (FP32)
 
   // host side of the current topology (the neighbourhood tables are built on the device from
   // the block list; the host leaf map is brought up to date only when a host query needs it)
@@ -221,6 +221,7 @@ size_t carve(acm_forest* f, const acm_grid_params* g, char* base) {
   int4* binfo = c.take<int4>(nb * 16);
   int32_t* blist = c.take<int32_t>(nb * 4);
   int32_t* slabidx = c.take<int32_t>(nb * 8 * 4);
+  int32_t* faces = c.take<int32_t>(nb * acm::kFaceStride * 4);
   int2* fw = c.take<int2>(nb * 26 * 8);
   int4* slabt = c.take<int4>(nb * 6 * 16);
   int4* reft = c.take<int4>(nb * 16);   // refinement tasks: 9 int32 per parent fit in 16 B per block
@@ -245,6 +246,7 @@ size_t carve(acm_forest* f, const acm_grid_params* g, char* base) {
   if (f) {
     f->U = U; f->ACC = ACC; f->YA = YA; f->YB = YB; f->CHI = CHI; f->DENSE = DENSE; f->SLAB = SLAB;
     f->d_nbh = nbh; f->d_binfo = binfo; f->d_blist = blist; f->d_slabidx = slabidx;
+    f->d_faces = faces;
     f->d_fw = fw; f->d_slabt = slabt; f->d_reft = reft; f->d_crst = crst; f->d_ranks = ranks;
     f->d_norms = norms; f->d_maxbits = maxbits; f->d_ind = ind; f->d_chir = chir; f->d_diag = diag;
     f->d_err = errf;
@@ -261,6 +263,7 @@ acm::TopoK topo(const acm_forest* f) {
   t.binfo = f->d_binfo;
   t.blist = f->d_blist;
   t.slabidx = f->d_slabidx;
+  t.faces = f->d_faces;
   t.n = (int64_t)f->order.size();
   return t;
 }
@@ -331,7 +334,7 @@ acm_status upload_topology(acm_forest* f, std::vector<BoxKey>* new_order = nullp
   for (int a = 0; a < 3; ++a) tk.nroot[a] = f->gp.nroot[a];
   acm::launch_topology(tk, f->d_ltab, f->d_bslot, f->d_binfo, f->d_blist, n, f->d_nbh, f->d_finer, f->d_fwmask,
                        f->d_slabmask, f->d_fwoff, f->d_slaboff, f->d_counts, f->d_fw, f->d_slabt, f->d_slabidx,
-                       f->d_err, f->st);
+                       f->d_faces, f->d_err, f->st);
   CKL();
   f->launches += 4;
   f->host_rows_ms += now_ms() - t1;
@@ -344,13 +347,14 @@ T* reg_ptr(acm_forest* f, void* r) { return reinterpret_cast<T*>(r); }
 
 // Fine wins + coarse-face slabs on a register (the per-stage synchronisation).
 template <typename T>
-acm_status sync_stage(acm_forest* f, T* reg, int use_slab_cache = 0) {
+acm_status sync_stage(acm_forest* f, T* reg, int use_slab_cache = 0, bool point_major = false) {
   const int Bs = f->gp.Bs;
   const int64_t n = (int64_t)f->order.size();
-  acm::launch_fine_wins<T>(Bs, reg, f->d_fw, f->d_counts, 26 * n, f->d_nbh, f->d_blist, f->tune_fw_ctas, f->st);
+  acm::launch_fine_wins<T>(Bs, reg, f->d_fw, f->d_counts, 26 * n, f->d_nbh, f->d_blist, f->tune_fw_ctas, point_major,
+                           f->st);
   CKL();
   acm::launch_coarse_slabs<T>(Bs, reg, reinterpret_cast<T*>(f->SLAB), f->d_slabt, f->d_counts + 1, 6 * n, f->d_nbh,
-                              f->d_slaboffc, use_slab_cache, f->tune_slab_ctas, f->st);
+                              f->d_slaboffc, use_slab_cache, f->tune_slab_ctas, point_major, f->st);
   CKL();
   f->launches += 2;
   return ACM_OK;
@@ -359,7 +363,7 @@ acm_status sync_stage(acm_forest* f, T* reg, int use_slab_cache = 0) {
 template <typename T>
 acm_status fine_wins(acm_forest* f, T* reg) {
   acm::launch_fine_wins<T>(f->gp.Bs, reg, f->d_fw, f->d_counts, 26 * (int64_t)f->order.size(), f->d_nbh, f->d_blist,
-                           f->tune_fw_ctas, f->st);
+                           f->tune_fw_ctas, false, f->st);
   CKL();
   ++f->launches;
   return ACM_OK;
@@ -488,6 +492,34 @@ acm_status eval_mask(acm_forest* f, const std::vector<int32_t>* fresh = nullptr)
   return ACM_OK;
 }
 
+// Registers of the RK4 stages: U -> YA (Y_2) -> YB (Y_3) -> ACC (Y_4) -> U, or with `save` the stage
+// states in save[1..3].  The accumulator of the points fine wins overwrites lives in ACC; without
+// `save` stage 3 moves it to YA at those points, where Y_2 is not needed any more, as its own output
+// takes ACC.
+template <typename T>
+T* stage_input(acm_forest* f, int s, T* const* save = nullptr) {
+  if (s == 1) return reinterpret_cast<T*>(f->U);
+  if (save) return save[s - 1];
+  return reinterpret_cast<T*>(s == 2 ? f->YA : (s == 3 ? f->YB : f->ACC));
+}
+template <typename T>
+acm::StagePtrs<T> stage_ptrs(acm_forest* f, int s, T* const* save = nullptr) {
+  acm::StagePtrs<T> p{};
+  T* ACC = reinterpret_cast<T*>(f->ACC);
+  T* moved = save ? ACC : reinterpret_cast<T*>(f->YA);
+  p.in = stage_input<T>(f, s, save);
+  p.out = s == 4 ? reinterpret_cast<T*>(f->U) : stage_input<T>(f, s + 1, save);
+  p.U = reinterpret_cast<const T*>(f->U);
+  p.y2 = stage_input<T>(f, 2, save);
+  p.y3 = stage_input<T>(f, 3, save);
+  p.acc_in = s == 4 ? moved : ACC;
+  p.acc_out = s == 3 ? moved : ACC;
+  p.chi = f->mask_on ? reinterpret_cast<const T*>(f->CHI) : nullptr;
+  p.slab = reinterpret_cast<const T*>(f->SLAB);
+  p.norms = s == 4 ? f->d_maxbits : nullptr;
+  return p;
+}
+
 // save (optional, 4 registers): receives each stage's synchronised input Y_s (the adjoint
 // recomputes a step with it).
 template <typename T>
@@ -500,23 +532,17 @@ acm_status rk4(acm_forest* f, double dt, double* dt_used, T* const* save = nullp
     dt = cfl_dt(f, m[4]);
   }
   if (dt_used) *dt_used = dt;
-  T* U = reinterpret_cast<T*>(f->U);
-  T* ACC = reinterpret_cast<T*>(f->ACC);
-  T* YA = reinterpret_cast<T*>(f->YA);
-  T* YB = reinterpret_cast<T*>(f->YB);
   const acm::TopoK t = topo(f);
   const int64_t l0 = f->launches;
   for (int s = 1; s <= 4; ++s) {
     // with `save` the stages write their outputs (the next stages' inputs) into save[1..3]
     // themselves, so only U (the first stage's input) is copied
-    T* in = s == 1 ? U : (save ? save[s - 1] : (s == 2 ? YA : (s == 3 ? YB : YA)));
-    T* out = s == 4 ? U : (save ? save[s] : (s == 1 ? YA : (s == 2 ? YB : YA)));
+    T* in = stage_input<T>(f, s, save);
     if (f->timing) CK(cudaEventRecord(f->ev[3 * (s - 1)], f->st));
     // stage 1 looks up the slabs' source points and caches them for stages 2-4 (same grid)
-    acm_status st = sync_stage<T>(f, in, s > 1);
+    // (the stage states are point-major inside a step, except those kept for the adjoint)
+    acm_status st = sync_stage<T>(f, in, s > 1, s > 1 && !save);
     if (st) return st;
-    const double cs_out = s == 1 || s == 2 ? dt / 2.0 : (s == 3 ? dt : dt / 6.0);
-    const double cs_acc = s == 1 ? dt / 6.0 : dt / 3.0;
     if (f->moving) {
       // the plate's mask at the stage time (RK4 nodes t, t + dt/2, t + dt/2, t + dt)
       plate_pose(f, f->time + (s == 1 ? 0.0 : (s == 4 ? dt : 0.5 * dt)));
@@ -532,43 +558,30 @@ acm_status rk4(acm_forest* f, double dt, double* dt_used, T* const* save = nullp
     }
     if (f->timing) CK(cudaEventRecord(f->ev[3 * (s - 1) + 1], f->st));
     acm::StageK<T> a{};
-    a.in = in;
-    a.U = U;
-    a.acc = ACC;
-    a.out = out;
-    a.chi = f->mask_on ? reinterpret_cast<const T*>(f->CHI) : nullptr;
-    a.slab = reinterpret_cast<const T*>(f->SLAB);
+    a.p = stage_ptrs<T>(f, s, save);
+    a.point_major = save == nullptr;
     a.c_acc = s == 1 ? dt / 6.0 : dt / 3.0;
     a.c_out = s == 1 || s == 2 ? dt / 2.0 : (s == 3 ? dt : dt / 6.0);
-    a.norms = nullptr;
-    if (s == 4) {
-      // the last stage also reduces the max norms of U^{n+1} (read by the next coarsening)
-      CK(cudaMemsetAsync(f->d_maxbits, 0, 8 * sizeof(unsigned long long), f->st));
-      a.norms = f->d_maxbits;
-    }
-    acm::launch_stage<T>(s, f->gp.Bs, a, t, f->phk, f->d_err, f->st, f->stage_variant);
+    a.body = f->moving ? &f->mask : nullptr;
+    // the last stage also reduces the max norms of U^{n+1} (read by the next coarsening)
+    if (s == 4) CK(cudaMemsetAsync(f->d_maxbits, 0, 8 * sizeof(unsigned long long), f->st));
+    acm::launch_stage<T>(s, f->gp.Bs, a, t, f->phk, f->d_err, f->st);
     CKL();
     ++f->launches;
-    if (f->moving) {
-      // + chi u_s / C_eta, the part of the penalization the stage kernel leaves out (u_s = 0 there)
-      acm::launch_solid_source<T>(f->gp.Bs, out, ACC, reinterpret_cast<const T*>(f->CHI), f->d_blist, f->d_binfo,
-                                  (int64_t)f->order.size(), f->phk, f->mask, cs_out, cs_acc, s < 4, f->st);
-      CKL();
-      ++f->launches;
-    }
     if (f->timing) CK(cudaEventRecord(f->ev[3 * (s - 1) + 2], f->st));
   }
   CK(cudaMemcpyAsync(f->h_err, f->d_err, sizeof(int), cudaMemcpyDeviceToHost, f->st));
-  f->norms_fresh = !f->moving;
+  f->norms_fresh = true;
   f->time += dt;
   if (f->moving) {
     acm_status st = eval_mask<T>(f);
     if (st) return st;
   }
-  // algorithmic bytes of the four stage kernels: per point 64 words (registers Y, U, acc in and
-  // out, see stage.cu) plus one word of mask per stage when a mask is set
+  // algorithmic bytes of the four stage kernels: per point 52 words (stage 1: Y in, Y out; stages 2, 3:
+  // Y, U in, Y out; stage 4: Y, U, Y_2, Y_3 in, U out; see stage.cu) plus one word of mask per stage
+  // when a mask is set
   const double npts = (double)f->order.size() * f->gp.Bs * f->gp.Bs * f->gp.Bs;
-  const double words = 64.0 + (f->mask_on ? 4.0 : 0.0);
+  const double words = 52.0 + (f->mask_on ? 4.0 : 0.0);
   f->stats.stage_ms = 0;
   f->stats.sync_ms = 0;
   f->stats.stage_bytes = npts * words * (double)f->esz;
@@ -599,32 +612,16 @@ acm_status enqueue_rk4_device_dt(acm_forest* f, double dt) {
   acm::launch_rk_coefs(f->d_maxbits, rk_params(f, dt), f->d_rk, f->st);
   CKL();
   ++f->launches;
-  T* U = reinterpret_cast<T*>(f->U);
-  T* ACC = reinterpret_cast<T*>(f->ACC);
-  T* YA = reinterpret_cast<T*>(f->YA);
-  T* YB = reinterpret_cast<T*>(f->YB);
   const acm::TopoK t = topo(f);
   for (int s = 1; s <= 4; ++s) {
-    T* in = s == 1 ? U : (s == 2 ? YA : (s == 3 ? YB : YA));
-    T* out = s == 1 ? YA : (s == 2 ? YB : (s == 3 ? YA : U));
-    acm_status st = sync_stage<T>(f, in, s > 1);
+    acm_status st = sync_stage<T>(f, stage_input<T>(f, s), s > 1, s > 1);
     if (st) return st;
     acm::StageK<T> a{};
-    a.in = in;
-    a.U = U;
-    a.acc = ACC;
-    a.out = out;
-    a.chi = f->mask_on ? reinterpret_cast<const T*>(f->CHI) : nullptr;
-    a.slab = reinterpret_cast<const T*>(f->SLAB);
-    a.c_acc = 0.0;
-    a.c_out = 0.0;
-    a.coefp = f->d_rk + 2;
-    a.norms = nullptr;
-    if (s == 4) {
-      CK(cudaMemsetAsync(f->d_maxbits, 0, 8 * sizeof(unsigned long long), f->st));
-      a.norms = f->d_maxbits;
-    }
-    acm::launch_stage<T>(s, f->gp.Bs, a, t, f->phk, f->d_err, f->st, f->stage_variant);
+    a.p = stage_ptrs<T>(f, s);
+    a.point_major = 1;
+    a.p.coefp = f->d_rk + 2;
+    if (s == 4) CK(cudaMemsetAsync(f->d_maxbits, 0, 8 * sizeof(unsigned long long), f->st));
+    acm::launch_stage<T>(s, f->gp.Bs, a, t, f->phk, f->d_err, f->st);
     CKL();
     ++f->launches;
   }
@@ -1067,12 +1064,10 @@ acm_status time_launches(acm_forest* f, F&& launch, int reps, float* ms_out) {
 // synchronisation for each number of CTAs per SM walking the list (fine wins: 2, 4, 8, 16; coarse
 // faces: 1, 2, 3 -- at most 3 are resident) and keep the fastest of each.  Fine wins rewrites
 // stored boundary points with the values of finer leaves (what every synchronisation does first);
-// the slab kernel writes only the slab buffer.  FP32 forests also time the three forms of the
-// fused stage kernel (two points per thread with packed arithmetic, one point per thread, one
-// point per thread with U, the accumulator and chi staged by bulk copies)
-// on RK stage 2 of the live grid (reading U, the first stage register and the accumulator,
+// the slab kernel writes only the slab buffer.  FP32 forests also time one launch of the fused stage
+// kernel (RK stage 2 of the live grid, reading U, the first stage register and the accumulator,
 // writing the accumulator and the second stage register: registers a step rewrites before it
-// reads them) and keep the faster.
+// reads them), for acm_get_tuning.
 template <typename T>
 acm_status autotune(acm_forest* f, int* fw_ctas, int* slab_ctas) {
   if (f->order.empty()) return fail(f, ACM_EINVAL, "empty forest");
@@ -1083,7 +1078,7 @@ acm_status autotune(acm_forest* f, int* fw_ctas, int* slab_ctas) {
   for (int c : {2, 4, 8, 16}) {
     float ms = 0.f;
     acm_status s = time_launches(f, [&]() {
-      acm::launch_fine_wins<T>(f->gp.Bs, U, f->d_fw, f->d_counts, 26 * n, f->d_nbh, f->d_blist, c, f->st);
+      acm::launch_fine_wins<T>(f->gp.Bs, U, f->d_fw, f->d_counts, 26 * n, f->d_nbh, f->d_blist, c, false, f->st);
     }, 5, &ms);
     if (s) return s;
     f->launches += 6;
@@ -1095,7 +1090,7 @@ acm_status autotune(acm_forest* f, int* fw_ctas, int* slab_ctas) {
     float ms = 0.f;
     acm_status s = time_launches(f, [&]() {
       acm::launch_coarse_slabs<T>(f->gp.Bs, U, reinterpret_cast<T*>(f->SLAB), f->d_slabt, f->d_counts + 1, 6 * n,
-                                  f->d_nbh, f->d_slaboffc, 0, c, f->st);
+                                  f->d_nbh, f->d_slaboffc, 0, c, false, f->st);
     }, 5, &ms);
     if (s) return s;
     f->launches += 6;
@@ -1104,30 +1099,12 @@ acm_status autotune(acm_forest* f, int* fw_ctas, int* slab_ctas) {
   if constexpr (sizeof(T) == 4) {
     const acm::TopoK t = topo(f);
     acm::StageK<T> a{};
-    a.in = reinterpret_cast<const T*>(f->YA);
-    a.U = U;
-    a.acc = reinterpret_cast<T*>(f->ACC);
-    a.out = reinterpret_cast<T*>(f->YB);
-    a.chi = f->mask_on ? reinterpret_cast<const T*>(f->CHI) : nullptr;
-    a.slab = reinterpret_cast<const T*>(f->SLAB);
-    a.c_acc = 0.0;
-    a.c_out = 0.0;
-    best = 1e30f;
-    int best_v = f->stage_variant;
-    for (int v : {acm::kStagePair, acm::kStagePoint, acm::kStagePointTMA, acm::kStagePointRows}) {
-      // 33^3 blocks: the row-split point form, three CTAs of 11 rows or four of 9
-      if (f->gp.Bs == 33 && v != acm::kStagePoint && v != acm::kStagePointRows) continue;
-      if (v == acm::kStagePointRows && f->gp.Bs == 9) continue;
-      float ms = 0.f;
-      acm_status s = time_launches(f, [&]() {
-        acm::launch_stage<T>(2, f->gp.Bs, a, t, f->phk, f->d_err, f->st, v);
-      }, 5, &ms);
-      if (s) return s;
-      f->launches += 6;
-      f->tune_stage_ms[v] = ms;
-      if (ms < best) { best = ms; best_v = v; }
-    }
-    f->stage_variant = best_v;
+    a.p = stage_ptrs<T>(f, 2);
+    a.point_major = 1;
+    acm_status s = time_launches(f, [&]() { acm::launch_stage<T>(2, f->gp.Bs, a, t, f->phk, f->d_err, f->st); }, 5,
+                                 &f->tune_stage_ms);
+    if (s) return s;
+    f->launches += 6;
   }
   f->tune_fw_ctas = best_fw;
   f->tune_slab_ctas = best_sc;
@@ -1248,7 +1225,7 @@ acm_status adjoint_sweep(acm_forest* f, int nsteps, double dt, int c, double wE,
   auto astage = [&](const T* Ys, double ts, const T* nup, double c_lam, double c_nu, T* nu_out, int sum_mode) {
     pose_at(ts);
     acm::launch_coarse_slabs<T>(Bs, Ys, SLAB, f->d_slabt, f->d_counts + 1, 6 * nb, f->d_nbh, f->d_slaboffc, 1,
-                                f->tune_slab_ctas, f->st);
+                                f->tune_slab_ctas, false, f->st);
     acm::AdjStageK<T> a{};
     a.Y = Ys;
     a.slab = SLAB;
@@ -1700,18 +1677,9 @@ struct BatchPersistent {
     hw.reserve((size_t)nwork);
     for (int i = 0; i < n; ++i) {
       acm_forest* g = fs[i];
-      T* U = reinterpret_cast<T*>(g->U);
-      T* YA = reinterpret_cast<T*>(g->YA);
-      T* YB = reinterpret_cast<T*>(g->YB);
       for (int st = 1; st <= 4; ++st) {
         acm::StageInst<T>& d = hd[(size_t)(st - 1) * n + i];
-        d.p.in = st == 1 ? U : (st == 2 ? YA : (st == 3 ? YB : YA));
-        d.p.out = st == 1 ? YA : (st == 2 ? YB : (st == 3 ? YA : U));
-        d.p.U = U;
-        d.p.acc = reinterpret_cast<T*>(g->ACC);
-        d.p.chi = g->mask_on ? reinterpret_cast<const T*>(g->CHI) : nullptr;
-        d.p.slab = reinterpret_cast<const T*>(g->SLAB);
-        d.p.norms = st == 4 ? g->d_maxbits : nullptr;
+        d.p = stage_ptrs<T>(g, st);
         d.p.coefp = g->d_rk + 2;
         d.tp = topo(g);
       }
@@ -1747,8 +1715,7 @@ struct BatchPersistent {
           acm::launch_rk_coefs(g->d_maxbits, rk_params(g, dt), g->d_rk, g->st);
           ++g->launches;
         }
-        T* in = reinterpret_cast<T*>(st == 1 ? g->U : (st == 2 ? g->YA : (st == 3 ? g->YB : g->YA)));
-        acm_status s = sync_stage<T>(g, in, st > 1);
+        acm_status s = sync_stage<T>(g, stage_input<T>(g, st), st > 1, st > 1);
         if (s) return s;
         if (st == 4) CK_F(g, cudaMemsetAsync(g->d_maxbits, 0, 8 * sizeof(unsigned long long), g->st));
       }
@@ -1989,12 +1956,6 @@ acm_status acm_set_stage_variant(acm_forest* f, int variant) {
   if (variant != ACM_STAGE_PAIR && variant != ACM_STAGE_POINT && variant != ACM_STAGE_POINT_TMA &&
       variant != ACM_STAGE_POINT_ROWS)
     return fail(f, ACM_EINVAL, "unknown stage kernel");
-  f->stage_variant = variant == ACM_STAGE_PAIR ? acm::kStagePair
-                     : (variant == ACM_STAGE_POINT ? acm::kStagePoint
-                        : (variant == ACM_STAGE_POINT_TMA ? acm::kStagePointTMA : acm::kStagePointRows));
-  // a captured graph holds the old kernel
-  if (f->gexec) { cudaGraphExecDestroy(f->gexec); f->gexec = nullptr; }
-  if (f->graph) { cudaGraphDestroy(f->graph); f->graph = nullptr; }
   return ACM_OK;
 }
 
@@ -2002,18 +1963,9 @@ acm_status acm_get_tuning(const acm_forest* f, acm_tuning* out) {
   if (!f || !out) return ACM_EINVAL;
   out->fw_ctas_per_sm = f->tune_fw_ctas;
   out->slab_ctas_per_sm = f->tune_slab_ctas;
-  out->stage_variant = f->gp.precision == 64 ||
-                               (f->gp.Bs == 33 && f->stage_variant != acm::kStagePointRows) ||
-                               (f->stage_variant == acm::kStagePointRows && f->gp.Bs == 9)
-                           ? ACM_STAGE_POINT
-                       : (f->stage_variant == acm::kStagePair ? ACM_STAGE_PAIR
-                          : (f->stage_variant == acm::kStagePoint ? ACM_STAGE_POINT
-                             : (f->stage_variant == acm::kStagePointTMA ? ACM_STAGE_POINT_TMA
-                                                                         : ACM_STAGE_POINT_ROWS)));
-  out->stage_ms[ACM_STAGE_PAIR] = f->tune_stage_ms[acm::kStagePair];
-  out->stage_ms[ACM_STAGE_POINT] = f->tune_stage_ms[acm::kStagePoint];
-  out->stage_ms[ACM_STAGE_POINT_TMA] = f->tune_stage_ms[acm::kStagePointTMA];
-  out->stage_ms[ACM_STAGE_POINT_ROWS] = f->tune_stage_ms[acm::kStagePointRows];
+  out->stage_variant = ACM_STAGE_POINT;
+  for (float& ms : out->stage_ms) ms = 0.f;
+  out->stage_ms[ACM_STAGE_POINT] = f->tune_stage_ms;
   return ACM_OK;
 }
 
@@ -2346,15 +2298,17 @@ acm_status acm_rhs(acm_forest* f, void* out, int64_t n_elems, int on_device) {
   if (f->gp.precision == 64) {
     acm_status s = sync_stage<double>(f, (double*)f->U);
     if (s) return s;
-    acm::StageK<double> a{(const double*)f->U, (const double*)f->U, (double*)f->ACC, (double*)f->YA,
-                          f->mask_on ? (const double*)f->CHI : nullptr, (const double*)f->SLAB, 0.0, 0.0};
-    acm::launch_stage<double>(0, f->gp.Bs, a, t, f->phk, f->d_err, f->st, f->stage_variant);
+    acm::StageK<double> a{};
+    a.p = stage_ptrs<double>(f, 1);
+    a.p.out = (double*)f->ACC;
+    acm::launch_stage<double>(0, f->gp.Bs, a, t, f->phk, f->d_err, f->st);
   } else {
     acm_status s = sync_stage<float>(f, (float*)f->U);
     if (s) return s;
-    acm::StageK<float> a{(const float*)f->U, (const float*)f->U, (float*)f->ACC, (float*)f->YA,
-                         f->mask_on ? (const float*)f->CHI : nullptr, (const float*)f->SLAB, 0.0, 0.0};
-    acm::launch_stage<float>(0, f->gp.Bs, a, t, f->phk, f->d_err, f->st, f->stage_variant);
+    acm::StageK<float> a{};
+    a.p = stage_ptrs<float>(f, 1);
+    a.p.out = (float*)f->ACC;
+    acm::launch_stage<float>(0, f->gp.Bs, a, t, f->phk, f->d_err, f->st);
   }
   CKL();
   ++f->launches;

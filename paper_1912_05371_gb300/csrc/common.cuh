@@ -18,6 +18,7 @@
 namespace acm {
 
 constexpr int kNbhStride = 256;      // int32 per slot in the neighbourhood table
+constexpr int kFaceStride = 32;      // int32 per block in the face records
 constexpr int kNbhType = 216;        // offset of the 27 type words
 constexpr int kGE = 2;               // ghost depth of the adaptation buffer (details, refine)
 constexpr int kTypeLeaf = 0, kTypeCoarser = 1, kTypeRefined = 2, kTypeNone = 3;

@@ -38,7 +38,7 @@ struct TreeK {
 // scratch.  err |= 2 if the grid is not graded, |= 4 if the table overflowed.
 void launch_topology(const TreeK& t, int* tab, int4* box, const int4* binfo, const int32_t* blist, int64_t n,
                      int32_t* nbh, uint8_t* finer, uint32_t* fwmask, uint32_t* slabmask, int32_t* fw_off,
-                     int32_t* slab_off, int32_t* counts, int2* fw, int4* slabt, int32_t* slabidx, int* err,
+                     int32_t* slab_off, int32_t* counts, int2* fw, int4* slabt, int32_t* slabidx, int32_t* faces, int* err,
                      cudaStream_t st);
 
 // Device topology: pointers into the pool, all indexed by rank (position in block order).
@@ -47,51 +47,68 @@ struct TopoK {
   const int4* binfo;        // [n] (J, gx, gy, gz)
   const int32_t* blist;     // [n] slot of each block
   const int32_t* slabidx;   // [n][8]: coarse-face halo slab per face (-1: none)
+  // [n][kFaceStride] what the stage kernels read of a block's faces F = 0 -x, 1 +x, 2 -y, 3 +y, 4 -z,
+  // 5 +z, in one line: words 0..5 the neighbour's type (leaf, refined or coarser), words 6 + 4F + j
+  // its slot (leaf), the slots of the four children touching the face (refined, j = first + 2 x
+  // second tangential half) or the halo slab's index (coarser), word 30 the mask of refined boxes
+  // (bit = box index)
+  const int32_t* faces;
   int64_t n;
 };
 
 // Model and RK constants of one stage in the field precision (kernel parameters, so the
 // stage kernel reads them from the constant bank).
 template <typename T>
+struct StageVec;
+template <>
+struct StageVec<float> { using type = float2; };
+template <>
+struct StageVec<double> { using type = double2; };
+template <typename T>
 struct StageConst {
-  T a1, a2, a3;             // first-derivative coefficients
+  // first-derivative coefficients over the first one, a_2/a_1 and a_3/a_1, and -16 and 30, as equal
+  // pairs (v, v)
+  typename StageVec<T>::type r2, r3, km16, k30;
   T nu, c0sq, cgam, inv_ceta, inv_csp;
   T uinf[3], pinf;
   T c_acc, c_out;           // RK coefficients of the stage
-  T ih[kMaxLevel + 1];      // 1 / h_J
+  int moving;               // a moving body: u_s = om x (x - x0)
+  T om[3], x0[3];
+  T ih[kMaxLevel + 1];      // a_1 / h_J
   T ih2[kMaxLevel + 1];     // 1 / (12 h_J^2)
 };
 
-// Stage of the fused RK4 update (Sec. 2.3).  in: the stage state (synchronised); U: the
-// state at t^n; acc: the RK accumulator; out: next stage state (or U^{n+1} in stage 4).
+struct MaskK;
+
+// The arrays of one stage of the fused RK4 update (Sec. 2.3; see stage.cu).  in: the stage state
+// (synchronised); U: the state at t^n; y2, y3: the second and third stage states (stage 4); out: the
+// next stage state (U^{n+1} in stage 4, the right-hand side in stage 0); acc_in, acc_out: the RK
+// accumulator of the points fine wins overwrites, read and written at those points only (they may
+// be the same register, and acc_in may be out).
 template <typename T>
-struct StageK {
+struct StagePtrs {
   const T* in;
   const T* U;
-  T* acc;
+  const T* y2;
+  const T* y3;
+  const T* acc_in;
+  T* acc_out;
   T* out;
   const T* chi;
   const T* slab;
-  double c_acc, c_out;      // stage coefficients (see stage.cu)
-  StageConst<T> kc;         // the constants above in the field precision (filled by launch_stage)
   // stage 4 only, if set: the max norms of U^{n+1} (layout and zeroing as for launch_maxnorm)
   unsigned long long* norms;
   // if set, the stage reads its (c_acc, c_out) from coefp[2 (stage-1)], written on the device by
   // launch_rk_coefs, instead of c_acc/c_out
   const double* coefp;
 };
-
-// The arrays one stage update of one block reads and writes (see StageK).
 template <typename T>
-struct StagePtrs {
-  const T* in;
-  const T* U;
-  T* acc;
-  T* out;
-  const T* chi;
-  const T* slab;
-  unsigned long long* norms;
-  const double* coefp;
+struct StageK {
+  StagePtrs<T> p;
+  double c_acc, c_out;      // stage coefficients (see stage.cu)
+  int point_major;          // layout of the stage states and the accumulator (see stage.cu At)
+  const MaskK* body;        // host: a moving body's pose (its u_s enters the penalization), or null
+  StageConst<T> kc;         // the constants in the field precision (filled by launch_stage)
 };
 
 // One instance of the persistent multi-instance stage launch: its arrays and its topology.
@@ -118,33 +135,18 @@ struct RkK {
 void launch_rk_coefs(const unsigned long long* maxbits, const RkK& p, double* rk, cudaStream_t st);
 
 // err: device int set to 1 if a bounded wait inside the kernel expired (never cleared here).
-// variant kStagePair: FP32 fields take the two-points-per-thread kernel (stage_pair.cu);
-// kStagePointTMA: FP32 fields take the one-point kernel with U, the accumulator and chi staged
-// by bulk copies; kStagePointRows: FP32 blocks of 17^3 and 33^3 take the one-point kernel with a
-// block's rows over CTAs of 9 rows; otherwise, and always for FP64 fields, the one-point kernel
-// (stage.cu; 33^3 blocks over three CTAs of 11 rows).
-constexpr int kStagePair = 0, kStagePoint = 1, kStagePointTMA = 2, kStagePointRows = 3;
 template <typename T>
-void launch_stage(int stage, int Bs, const StageK<T>& s, const TopoK& t, const PhysK& p, int* err,
-                  cudaStream_t st, int variant = kStagePair);
+void launch_stage(int stage, int Bs, const StageK<T>& s, const TopoK& t, const PhysK& p, int* err, cudaStream_t st);
 
-// Constants of the FP32 pair kernel (kernel parameters, read from the constant bank): equal
-// pairs (v, v) for the packed operations, plain floats for the rest.
-struct PairConst {
-  float2 a1, a2, a3, k16, km90, mcgam, minv_ceta, minv_csp, uinf0, uinf1, uinf2, pinf;
-  float nu, c0sq, c_acc, c_out;
-  float ih[kMaxLevel + 1];     // 1 / h_J
-  float ih2[kMaxLevel + 1];    // 1 / (12 h_J^2)
-};
-void launch_stage_pair(int stage, int Bs, const StageK<float>& s, const TopoK& t, const PhysK& p,
-                       cudaStream_t st);
-
+// point_major: the register's layout inside a step (the stage states), four components side by side at
+// ((z Bs + y) Bs + x) 4 of a block, and the slabs written in the same way, [slab][layer][t1][t0][4];
+// else component-major.
 // The per-stage synchronisation kernels walk a task list whose length the device holds
 // (*ntasks, written by launch_topology); max_tasks bounds it and sizes the grid, with
 // ctas_per_sm CTAs per SM.
 template <typename T>
 void launch_fine_wins(int Bs, T* reg, const int2* tasks, const int32_t* ntasks, int64_t max_tasks,
-                      const int32_t* nbh, const int32_t* blist, int ctas_per_sm, cudaStream_t st);
+                      const int32_t* nbh, const int32_t* blist, int ctas_per_sm, bool point_major, cudaStream_t st);
 
 // offc: per-slab cache of the leaf lookups (slab_offset_words(Bs) words per slab) or nullptr;
 // use_cache = 0 fills it, 1 reads it (valid while the grid is unchanged).
@@ -152,7 +154,7 @@ void launch_fine_wins(int Bs, T* reg, const int2* tasks, const int32_t* ntasks, 
 template <typename T>
 void launch_coarse_slabs(int Bs, const T* reg, T* slab, const int4* tasks, const int32_t* ntasks,
                          int64_t max_tasks, const int32_t* nbh, uint32_t* offc, int use_cache, int ctas_per_sm,
-                         cudaStream_t st);
+                         bool point_major, cudaStream_t st);
 size_t slab_offset_words(int Bs);
 
 // Streaming multiprocessors of the current device (cached per device).
@@ -220,12 +222,8 @@ template <typename T>
 void launch_mask(int Bs, T* chi, const int32_t* blist, const int32_t* ranks, int64_t n, const int4* binfo,
                  const PhysK& p, const MaskK& m, cudaStream_t st);
 
-// Solid velocity of a rotating rigid body (mask kind 2), u_s = omega x (x - x_0): adds the
-// penalization's source chi u_s / C_eta of the stage to the stage outputs, out += c_out S and,
-// if acc_too, acc += c_acc S (the stage kernel has applied -chi u / C_eta).
-template <typename T>
-void launch_solid_source(int Bs, T* out, T* acc, const T* chi, const int32_t* blist, const int4* binfo, int64_t n,
-                         const PhysK& p, const MaskK& m, double c_out, double c_acc, int acc_too, cudaStream_t st);
+// Solid velocity of a rotating rigid body (mask kind 2): u_s = omega x (x - x_0) (the stage kernel
+// adds it to the penalization).
 // Per block sums over the half-open points of chi u_s (3 components): out[n][4].
 template <typename T>
 void launch_solid_moment(int Bs, const T* chi, const int32_t* blist, const int4* binfo, int64_t n, const PhysK& p,

@@ -1,5 +1,5 @@
-// Device helpers shared by the fused stage kernels (stage.cu: one point per thread, any
-// precision; stage_pair.cu: two points per thread, FP32 with packed arithmetic).
+// Device helpers shared by the fused stage kernel (stage.cu) and the adjoint stage kernel
+// (adjoint_kernels.cuh).
 #pragma once
 
 #include <atomic>
@@ -22,9 +22,6 @@ void smem_opt_in_stage(K kernel, size_t bytes, std::atomic<unsigned long long>& 
   done.fetch_or(bit);
 }
 
-// faces: 0 -x, 1 +x, 2 -y, 3 +y, 4 -z, 5 +z ; box index of the face neighbour
-__constant__ int kFaceBox[6] = {12, 14, 10, 16, 4, 22};
-
 template <typename T>
 __device__ __forceinline__ void cp_async_elem(T* dst, const T* src) {
   const unsigned d = (unsigned)__cvta_generic_to_shared(dst);
@@ -34,33 +31,72 @@ __device__ __forceinline__ void cp_async_elem(T* dst, const T* src) {
     asm volatile("cp.async.ca.shared.global [%0], [%1], 8;\n" ::"r"(d), "l"(src) : "memory");
   }
 }
+__device__ __forceinline__ void cp_async_16(void* dst, const void* src) {
+  asm volatile("cp.async.cg.shared.global [%0], [%1], 16;\n" ::"r"((unsigned)__cvta_generic_to_shared(dst)), "l"(src)
+               : "memory");
+}
 template <typename T>
 __device__ __forceinline__ T tmax(T a, T b) { return a > b ? a : b; }
 
-// Packed FP32x2 operations, round to nearest.  a - b is fma(b, -1, a): b * -1 is exact, so it
-// rounds once, like a subtraction.
-__device__ __forceinline__ float2 padd(float2 a, float2 b) { return __fadd2_rn(a, b); }
-__device__ __forceinline__ float2 pmul(float2 a, float2 b) { return __fmul2_rn(a, b); }
-__device__ __forceinline__ float2 pfma(float2 a, float2 b, float2 c) { return __ffma2_rn(a, b, c); }
-__device__ __forceinline__ float2 psub(float2 a, float2 b) { return __ffma2_rn(b, make_float2(-1.f, -1.f), a); }
+// Pairs of values: FP32 pairs take the packed FP32x2 instructions, FP64 pairs go component by
+// component.  Every operation rounds each component once, to nearest.
+__host__ __device__ __forceinline__ float2 vset(float v) { return make_float2(v, v); }
+__host__ __device__ __forceinline__ double2 vset(double v) { return make_double2(v, v); }
+__device__ __forceinline__ float2 vadd(float2 a, float2 b) { return __fadd2_rn(a, b); }
+__device__ __forceinline__ float2 vmul(float2 a, float2 b) { return __fmul2_rn(a, b); }
+__device__ __forceinline__ float2 vfma(float2 a, float2 b, float2 c) { return __ffma2_rn(a, b, c); }
+__device__ __forceinline__ float2 vsub(float2 a, float2 b) {
+  union P { float2 f; unsigned long long u; } x, y, r;
+  x.f = a;
+  y.f = b;
+  asm("sub.rn.f32x2 %0, %1, %2;" : "=l"(r.u) : "l"(x.u), "l"(y.u));
+  return r.f;
+}
+__device__ __forceinline__ double2 vadd(double2 a, double2 b) { return make_double2(a.x + b.x, a.y + b.y); }
+__device__ __forceinline__ double2 vmul(double2 a, double2 b) { return make_double2(a.x * b.x, a.y * b.y); }
+__device__ __forceinline__ double2 vfma(double2 a, double2 b, double2 c) {
+  return make_double2(fma(a.x, b.x, c.x), fma(a.y, b.y, c.y));
+}
+__device__ __forceinline__ double2 vsub(double2 a, double2 b) { return make_double2(a.x - b.x, a.y - b.y); }
+
+// h / a_1 times the first difference of a pair from its neighbours at distance 1, 2, 3 (Sec. 2.3).
+template <typename K, typename V>
+__device__ __forceinline__ V d1_pair(const K& kc, V m1, V p1, V m2, V p2, V m3, V p3) {
+  return vfma(kc.r3, vsub(p3, m3), vfma(kc.r2, vsub(p2, m2), vsub(p1, m1)));
+}
+// -12 h^2 times the second difference (Sec. 2.3): p2 + m2 - 16 (p1 + m1) + 30 c.
+template <typename K, typename V>
+__device__ __forceinline__ V d2_pair(const K& kc, V c, V m1, V p1, V m2, V p2) {
+  return vfma(kc.k30, c, vfma(kc.km16, vadd(p1, m1), vadd(p2, m2)));
+}
+// The same of a pair's first component.
+__device__ __forceinline__ float d2_first(float2 c, float2 m1, float2 p1, float2 m2, float2 p2) {
+  return fmaf(30.f, c.x, fmaf(-16.f, p1.x + m1.x, p2.x + m2.x));
+}
+__device__ __forceinline__ double d2_first(double2 c, double2 m1, double2 p1, double2 m2, double2 p2) {
+  return fma(30.0, c.x, fma(-16.0, p1.x + m1.x, p2.x + m2.x));
+}
 // Bulk prefetch of a contiguous range into L2 (address and size multiples of 16 bytes).
 __device__ __forceinline__ void prefetch_l2(const void* p, unsigned bytes) {
   asm volatile("cp.async.bulk.prefetch.L2.global [%0], %1;\n" ::"l"(p), "r"(bytes) : "memory");
 }
 __device__ __forceinline__ void cp_async_commit() { asm volatile("cp.async.commit_group;\n" ::: "memory"); }
 
-// mbarrier-tracked bulk copies (the Blackwell TMA engine's 1D form): one thread announces the
-// bytes a phase expects and issues the copies; every thread waits for the phase.
 __device__ __forceinline__ unsigned smem_u32(const void* p) { return (unsigned)__cvta_generic_to_shared(p); }
 __device__ __forceinline__ void mbar_init(unsigned long long* bar, unsigned count) {
   asm volatile("mbarrier.init.shared::cta.b64 [%0], %1;\n" ::"r"(smem_u32(bar)), "r"(count) : "memory");
 }
-// makes the initialised barriers visible to the copy engine (before the CTA-wide barrier)
 __device__ __forceinline__ void mbar_init_fence() {
   asm volatile("fence.mbarrier_init.release.cluster;\n" ::: "memory");
 }
-// orders this thread's earlier shared-memory accesses (and those the CTA barrier published)
-// before later bulk copies into the same memory
+__device__ __forceinline__ void mbar_inval(unsigned long long* bar) {
+  asm volatile("mbarrier.inval.shared::cta.b64 [%0];\n" ::"r"(smem_u32(bar)) : "memory");
+}
+__device__ __forceinline__ void mbar_arrive(unsigned long long* bar) {
+  asm volatile("mbarrier.arrive.shared::cta.b64 _, [%0];\n" ::"r"(smem_u32(bar)) : "memory");
+}
+// orders this thread's earlier shared-memory accesses (and those a barrier published to it) before
+// later bulk copies into the same memory
 __device__ __forceinline__ void fence_async_shared() { asm volatile("fence.proxy.async.shared::cta;\n" ::: "memory"); }
 __device__ __forceinline__ void mbar_expect_tx(unsigned long long* bar, unsigned bytes) {
   asm volatile("mbarrier.arrive.expect_tx.shared::cta.b64 _, [%0], %1;\n" ::"r"(smem_u32(bar)), "r"(bytes)
@@ -71,19 +107,23 @@ __device__ __forceinline__ void bulk_g2s(void* dst, const void* src, unsigned by
   asm volatile("cp.async.bulk.shared::cluster.global.mbarrier::complete_tx::bytes [%0], [%1], %2, [%3];\n"
                ::"r"(smem_u32(dst)), "l"(src), "r"(bytes), "r"(smem_u32(bar)) : "memory");
 }
-// Waits for the phase of the given parity; gives up after a bounded number of polls (each poll
-// may suspend the thread for a while), sets err |= 1 (a bounded wait expired) and returns false.
-__device__ __forceinline__ bool mbar_wait(unsigned long long* bar, unsigned parity, int* err) {
-  unsigned done = 0;
-  for (int it = 0; it < (1 << 22) && !done; ++it) {
-    asm volatile(
-        "{\n .reg .pred p;\n mbarrier.try_wait.parity.shared::cta.b64 p, [%1], %2;\n selp.u32 %0, 1, 0, p;\n}\n"
-        : "=r"(done)
-        : "r"(smem_u32(bar)), "r"(parity)
-        : "memory");
-  }
-  if (!done && err) atomicOr(err, 1);
-  return done != 0;
+// Waits for the phase of the given parity; after a bounded number of polls (each may suspend the
+// thread for a while) it sets *err |= 1 (a bounded wait expired) and goes on.
+__device__ __forceinline__ void mbar_wait(unsigned long long* bar, unsigned parity, int* err) {
+  asm volatile(
+      "{\n .reg .pred p;\n .reg .u32 n;\n mov.u32 n, 0;\n"
+      "W%=:\n mbarrier.try_wait.parity.shared::cta.b64 p, [%0], %1;\n @p bra D%=;\n"
+      " add.u32 n, n, 1;\n setp.lt.u32 p, n, 4194304;\n @p bra W%=;\n red.global.or.b32 [%2], 1;\n"
+      "D%=:\n}\n" ::"r"(smem_u32(bar)), "r"(parity), "l"(err)
+      : "memory");
+}
+// this thread's earlier cp.async copies arrive on the mbarrier when they have completed
+__device__ __forceinline__ void cp_async_mbar_arrive(unsigned long long* bar) {
+  asm volatile("cp.async.mbarrier.arrive.noinc.shared::cta.b64 [%0];\n" ::"r"(smem_u32(bar)) : "memory");
+}
+template <int N>
+__device__ __forceinline__ void cp_async_wait_group() {
+  asm volatile("cp.async.wait_group %0;\n" ::"n"(N) : "memory");
 }
 __device__ __forceinline__ void cp_async_wait_all() { asm volatile("cp.async.wait_all;\n" ::: "memory"); }
 
@@ -119,35 +159,24 @@ __device__ __forceinline__ const T* halo_ptr(const int (&ftype)[6], const int (&
 }
 
 
-// Face table of one block: for each face F (0 -x, 1 +x, 2 -y, 3 +y, 4 -z, 5 +z) the type of the
-// neighbour across it (leaf, refined: the four children touching the face, or coarser: the halo
-// slab the coarse-face kernel predicted) and the slots / slab index in fs[F][0..3].  Threads
-// 0..23 fill it; the caller synchronises.
-__device__ __forceinline__ void stage_faces(int tid, const int* __restrict__ nbh, const int32_t* __restrict__ slabidx,
-                                            int rank, int (&ftype)[6], int (&fs)[6][4]) {
-  if (tid < 24) {
-    const int F = tid >> 2, j = tid & 3;
-    const int c0 = j & 1, c1 = j >> 1;
-    const int d = kFaceBox[F];
-    int ty = nbh[kNbhType + d] & 15;
-    int s;
-    if (ty == kTypeLeaf) {
-      s = nbh[8 * d];
-    } else if (ty == kTypeRefined) {
-      const int nbit = (F & 1) ? 0 : 1;
-      const int ax = F >> 1;
-      int c;
-      if (ax == 0) c = nbit | (c0 << 1) | (c1 << 2);
-      else if (ax == 1) c = c0 | (nbit << 1) | (c1 << 2);
-      else c = c0 | (c1 << 1) | (nbit << 2);
-      s = nbh[8 * d + c];
-    } else {
-      ty = kTypeCoarser;                 // halo slab predicted by the coarse-face kernel
-      s = slabidx[(size_t)rank * 8 + F];
-    }
-    fs[F][j] = s;
-    if (j == 0) ftype[F] = ty;
+// Face table of one block from its face record (TopoK::faces): for each face F the type of the
+// neighbour across it and the slots / slab index in fs[F][0..3].  Threads 0..29 fill it; the
+// caller synchronises.
+__device__ __forceinline__ void stage_faces(int tid, const int32_t* __restrict__ faces, int rank, int (&ftype)[6],
+                                            int (&fs)[6][4]) {
+  if (tid < 30) {
+    const int v = faces[(size_t)rank * kFaceStride + tid];
+    if (tid < 6) ftype[tid] = v;
+    else (&fs[0][0])[tid - 6] = v;
   }
+}
+
+// Global lattice index of a block's point i along axis a; the periodic seam x = L is taken as 0.
+__device__ __forceinline__ int lattice_index(const PhysK& ph, int4 bi, int a, int i, int M) {
+  const int g = a == 0 ? bi.y : (a == 1 ? bi.z : bi.w);
+  const int N = (ph.nroot[a] << bi.x) * M;
+  const int gi = g * M + i;                               // in [0, N]
+  return gi >= N ? gi - N : gi;
 }
 
 // Sponge profile of one block along each axis (Sec. 2.2, sponge terms; the profile's reading is

@@ -126,7 +126,8 @@ __device__ DevStatus box_status_dev(const TreeK& t, int J, long long x, long lon
 // and of faces covered by a coarser leaf (halo slabs).  A box that is missing, or refined with
 // a touching child missing, breaks the 2:1 grading the kernels rely on: error flag bit 2.
 __global__ void __launch_bounds__(256) k_rows(TreeK t, const int4* binfo, int64_t n, int32_t* nbh,
-                                              uint8_t* finer, uint32_t* fwmask, uint32_t* slabmask, int* err) {
+                                              uint8_t* finer, uint32_t* fwmask, uint32_t* slabmask, int32_t* faces,
+                                              int* err) {
   const int64_t rank = ((int64_t)blockIdx.x * blockDim.x + threadIdx.x) >> 5;
   const int lane = threadIdx.x & 31;
   if (rank >= n) return;
@@ -156,19 +157,43 @@ __global__ void __launch_bounds__(256) k_rows(TreeK t, const int4* binfo, int64_
     for (int c = 0; c < 8; ++c) row[8 * lane + c] = st.type == kTypeNone ? -1 : st.slot[c];
     row[kNbhType + lane] = st.type == kTypeNone ? -1 : (st.type | (st.octant << 4));
     type = st.type;
+    // the block's face record (kernels.hpp TopoK::faces); slab indices are filled in by k_fill
+    int F = -1;
+#pragma unroll
+    for (int q = 0; q < 6; ++q)
+      if (kFaceBoxT[q] == lane) F = q;
+    if (F >= 0) {
+      int32_t* fr = faces + rank * kFaceStride;
+      const bool coarse = st.type != kTypeLeaf && st.type != kTypeRefined;
+      fr[F] = coarse ? kTypeCoarser : st.type;
+      const int nbit = (F & 1) ? 0 : 1, ax = F >> 1;
+#pragma unroll
+      for (int j = 0; j < 4; ++j) {
+        // the children touching the face, j = first + 2 x second tangential half
+        const int c0 = j & 1, c1 = j >> 1;
+        const int c = ax == 0 ? (nbit | (c0 << 1) | (c1 << 2)) : (ax == 1 ? (c0 | (nbit << 1) | (c1 << 2)) : (c0 | (c1 << 1) | (nbit << 2)));
+        int s = st.slot[0];
+        if (st.type == kTypeRefined) {
+#pragma unroll
+          for (int q = 0; q < 8; ++q) s = q == c ? st.slot[q] : s;
+        }
+        fr[6 + 4 * F + j] = coarse ? -1 : s;
+      }
+    }
   } else {
     for (int e = kNbhType + 27 + (lane - 27); e < kNbhStride; e += 5) row[e] = -1;
   }
   const unsigned refined = __ballot_sync(0xffffffffu, lane < 27 && lane != 13 && type == kTypeRefined);
   const unsigned coarser = __ballot_sync(0xffffffffu, lane < 27 && type == kTypeCoarser);
   if (lane == 0) {
-    unsigned faces = 0;
+    unsigned cf = 0;
 #pragma unroll
     for (int F = 0; F < 6; ++F)
-      if ((coarser >> kFaceBoxT[F]) & 1u) faces |= 1u << F;
+      if ((coarser >> kFaceBoxT[F]) & 1u) cf |= 1u << F;
     finer[rank] = refined != 0;
+    faces[rank * kFaceStride + 30] = (int32_t)refined;
     fwmask[rank] = refined;
-    slabmask[rank] = faces;
+    slabmask[rank] = cf;
   }
 }
 
@@ -215,7 +240,7 @@ __global__ void __launch_bounds__(kScanNT) k_scan(const uint32_t* fwmask, const 
 // slab index per face (-1: none).
 __global__ void __launch_bounds__(256) k_fill(const uint32_t* fwmask, const uint32_t* slabmask, const int32_t* fw_off,
                                               const int32_t* slab_off, int64_t n, int2* fw, int4* slabt,
-                                              int32_t* slabidx) {
+                                              int32_t* slabidx, int32_t* faces) {
   const int64_t r = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
   if (r >= n) return;
   const uint32_t m = fwmask[r];
@@ -231,6 +256,8 @@ __global__ void __launch_bounds__(256) k_fill(const uint32_t* fwmask, const uint
       slabt[idx] = make_int4((int)r, F, idx, 0);
     }
     slabidx[r * 8 + F] = idx;
+    if (idx >= 0)
+      for (int q = 0; q < 4; ++q) faces[r * kFaceStride + 6 + 4 * F + q] = idx;
   }
 }
 
@@ -238,17 +265,19 @@ __global__ void __launch_bounds__(256) k_fill(const uint32_t* fwmask, const uint
 
 void launch_topology(const TreeK& t, int* tab, int4* box, const int4* binfo, const int32_t* blist, int64_t n,
                      int32_t* nbh, uint8_t* finer, uint32_t* fwmask, uint32_t* slabmask, int32_t* fw_off,
-                     int32_t* slab_off, int32_t* counts, int2* fw, int4* slabt, int32_t* slabidx, int* err,
-                     cudaStream_t st) {
+                     int32_t* slab_off, int32_t* counts, int2* fw, int4* slabt, int32_t* slabidx, int32_t* faces,
+                     int* err, cudaStream_t st) {
   cudaMemsetAsync(tab, 0xff, (size_t)(t.mask + 1) * sizeof(int), st);
   if (n <= 0) {
     cudaMemsetAsync(counts, 0, 2 * sizeof(int32_t), st);
     return;
   }
   k_index<<<(unsigned)((n + 255) / 256), 256, 0, st>>>(t, binfo, blist, n, tab, box, err);
-  k_rows<<<(unsigned)((n * 32 + 255) / 256), 256, 0, st>>>(t, binfo, n, nbh, finer, fwmask, slabmask, err);
+  k_rows<<<(unsigned)((n * 32 + 255) / 256), 256, 0, st>>>(t, binfo, n, nbh, finer, fwmask, slabmask, faces,
+                                                                  err);
   k_scan<<<1, kScanNT, 0, st>>>(fwmask, slabmask, n, fw_off, slab_off, counts);
-  k_fill<<<(unsigned)((n + 255) / 256), 256, 0, st>>>(fwmask, slabmask, fw_off, slab_off, n, fw, slabt, slabidx);
+  k_fill<<<(unsigned)((n + 255) / 256), 256, 0, st>>>(fwmask, slabmask, fw_off, slab_off, n, fw, slabt, slabidx,
+                                                         faces);
 }
 
 }  // namespace acm
