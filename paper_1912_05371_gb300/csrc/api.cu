@@ -608,7 +608,7 @@ acm::RkK rk_params(const acm_forest* f, double dt) {
 }
 
 template <typename T>
-acm_status enqueue_rk4_device_dt(acm_forest* f, double dt) {
+acm_status enqueue_rk4_device_dt(acm_forest* f, double dt, int64_t side_by_side = 0) {
   acm::launch_rk_coefs(f->d_maxbits, rk_params(f, dt), f->d_rk, f->st);
   CKL();
   ++f->launches;
@@ -619,6 +619,7 @@ acm_status enqueue_rk4_device_dt(acm_forest* f, double dt) {
     acm::StageK<T> a{};
     a.p = stage_ptrs<T>(f, s);
     a.point_major = 1;
+    a.side_by_side = side_by_side;
     a.p.coefp = f->d_rk + 2;
     if (s == 4) CK(cudaMemsetAsync(f->d_maxbits, 0, 8 * sizeof(unsigned long long), f->st));
     acm::launch_stage<T>(s, f->gp.Bs, a, t, f->phk, f->d_err, f->st);
@@ -1723,8 +1724,8 @@ struct BatchPersistent {
         CK_F(f0, cudaEventRecord(ev[i], forests[i]->st));
         CK_F(f0, cudaStreamWaitEvent(origin, ev[i], 0));
       }
-      acm::launch_stage_multi<T>(st, f0->gp.Bs, f0->phk, desc + (size_t)(st - 1) * n, work, nwork,
-                                 acm::sm_count() * 3, f0->d_err, origin);
+      acm::launch_stage_multi<T>(st, f0->gp.Bs, f0->phk, desc + (size_t)(st - 1) * n, work, nwork, f0->d_err,
+                                 origin);
       CK_F(f0, cudaGetLastError());
       ++f0->launches;
     }
@@ -1747,8 +1748,10 @@ acm_status acm_rk4_steps_batch(acm_forest* const* forests, int n, int nsteps, do
       if (forests[j] == forests[i]) return fail(forests[i], ACM_EINVAL, "forest listed twice");
   }
   if (nsteps == 0) return ACM_OK;
+  int64_t nblocks = 0;                    // the instances' steps run side by side
+  for (int i = 0; i < n; ++i) nblocks += (int64_t)forests[i]->order.size();
   auto step = [&](acm_forest* f) {
-    return f->gp.precision == 64 ? enqueue_rk4_device_dt<double>(f, dt) : enqueue_rk4_device_dt<float>(f, dt);
+    return f->gp.precision == 64 ? enqueue_rk4_device_dt<double>(f, dt, nblocks) : enqueue_rk4_device_dt<float>(f, dt, nblocks);
   };
   // the device clocks start from the host's; the first time step needs the norms of each U
   for (int i = 0; i < n; ++i) {

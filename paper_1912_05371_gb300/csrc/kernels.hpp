@@ -106,6 +106,7 @@ template <typename T>
 struct StageK {
   StagePtrs<T> p;
   double c_acc, c_out;      // stage coefficients (see stage.cu)
+  int64_t side_by_side;     // blocks that run at the same time on other streams included (0: this grid's)
   int point_major;          // layout of the stage states and the accumulator (see stage.cu At)
   const MaskK* body;        // host: a moving body's pose (its u_s enters the penalization), or null
   StageConst<T> kc;         // the constants in the field precision (filled by launch_stage)
@@ -118,13 +119,13 @@ struct StageInst {
   TopoK tp;
 };
 
-// One RK stage of several independent instances in one persistent launch (ctas CTAs walking the
+// One RK stage of several independent instances in one persistent launch (resident CTAs walking the
 // nwork (instance, rank) pairs of work); the instances share PhysK and take their stage
 // coefficients from their own p.coefp (the time step on the device).  desc and work are device
 // arrays.
 template <typename T>
 void launch_stage_multi(int stage, int Bs, const PhysK& p, const StageInst<T>* desc, const int2* work, int64_t nwork,
-                        int ctas, int* err, cudaStream_t st);
+                        int* err, cudaStream_t st);
 
 // Parameters of the device time step (Sec. 2.3): CFL rule as on the host; h = finest spacing.
 struct RkK {

@@ -306,13 +306,16 @@ __device__ __forceinline__ int fine_win_bits(unsigned m, int x, int y) {
   return (((m >> 9) & t) ? 1 : 0) | ((m & t) ? 2 : 0) | (((m >> 18) & t) ? 4 : 0);
 }
 
-// The update of one block (rank `rank` of the topology tp), rows part * RY .. of it; a: the
-// arrays, kc: the constants.
+// The update of one block (rank `rank` of the topology tp), rows of y part `part` and planes za .. ze - 1
+// of it; a: the arrays, kc: the constants.
 // MULTI: called again by the same CTA afterwards (the mbarriers are given back at the end).
 // PM: the stage states and the accumulator are point-major (see At); U is component-major.
-template <typename T, int BS, int STAGE, bool PM, bool MULTI>
+template <typename T, int BS, int STAGE, bool PM, bool MULTI, bool SPLIT>
 __device__ __forceinline__ void stage_block(const StagePtrs<T>& a, const StageConst<T>& kc, const TopoK& tp,
-                                            const PhysK& ph, int* err, const int rank, const int part) {
+                                            const PhysK& ph, int* err, const int rank, const int part,
+                                            const int za, const int ze) {
+  // (planes 0 .. M, known to the compiler, unless the block is split along z)
+  const int z0 = SPLIT ? za : 0, z1 = SPLIT ? ze : BS;
   using L = Lay<T, BS>;
   using C = Cfg<T, BS>;
   using V = typename StageVec<T>::type;
@@ -354,7 +357,7 @@ __device__ __forceinline__ void stage_block(const StagePtrs<T>& a, const StageCo
   const int x = act ? tid % BS : 0, y = y0 + (act ? tid / BS : 0);
   const size_t bo = (size_t)slot * L::BLK;
   const T* __restrict__ inb = a.in + bo;
-  // register ring: plane zz of the pencil sits in entry (zz + 3) % 7 (planes z - 3 .. z + 3 of
+  // register ring: plane zz of the pencil sits in entry (zz - z0 + 3) % 7 (planes z - 3 .. z + 3 of
   // iteration z; plane z + 3 enters at its start); the block's own planes are requested before the
   // first barrier, together with the face record
   V qa[7], qb[7];
@@ -362,7 +365,10 @@ __device__ __forceinline__ void stage_block(const StagePtrs<T>& a, const StageCo
   for (int k = 0; k < 7; ++k) qa[k] = qb[k] = vset(T(0));
   if (act) {
 #pragma unroll
-    for (int k = 3; k < 6; ++k) load_point<AI>(inb + I::idx(x, y, k - 3), I::CS, qa[k], qb[k]);
+    for (int k = SPLIT ? 0 : 3; k < 6; ++k) {
+      const int zz = z0 + k - 3;
+      if (!SPLIT || (zz >= 0 && zz <= M)) load_point<AI>(inb + I::idx(x, y, zz), I::CS, qa[k], qb[k]);
+    }
   }
   stage_sponge<T, BS>(tid, ph, bi, sp);
   if (tid == NT) {
@@ -397,11 +403,22 @@ __device__ __forceinline__ void stage_block(const StagePtrs<T>& a, const StageCo
     }
   };
   if (act) {
-    const T* p;
-    int ls, cs;
-    z_face(4, x, y, p, ls, cs);
+    if (!SPLIT || z0 < 3) {
+      const T* p;
+      int ls, cs;
+      z_face(4, x, y, p, ls, cs);
 #pragma unroll
-    for (int k = 0; k < 3; ++k) load_point<AI>(p + k * ls, cs, qa[2 - k], qb[2 - k]);
+      for (int k = 0; k < 3; ++k)         // plane z0 + k - 3, if below the block
+        if (z0 + k < 3) load_point<AI>(p + (2 - k - z0) * ls, cs, qa[k], qb[k]);
+    }
+    if (SPLIT && z0 + 2 > M) {
+      const T* p;
+      int ls, cs;
+      z_face(5, x, y, p, ls, cs);
+#pragma unroll
+      for (int k = 4; k < 6; ++k)         // plane z0 + k - 3, if above it
+        if (z0 + k - 3 > M) load_point<AI>(p + (z0 + k - 4 - M) * ls, cs, qa[k], qb[k]);
+    }
   }
   // x/y halo points of every plane as affine functions of z: component f of the point of plane z is
   // read at offset (z <= M/2 ? lo : hi) + z * hz + f * cs from the state (or from the slab buffer,
@@ -556,8 +573,9 @@ __device__ __forceinline__ void stage_block(const StagePtrs<T>& a, const StageCo
       if (src && (!is_in || z + 3 <= M))
         bulk_g2s(stg + ((size_t)sl * nst + lane) * SP, src + (size_t)z * pl, mine, &full[sl]);
     };
-    for (int z = 0; z < kND; ++z) fill(z, z);
-    if (C::CORNER && lane <= M) {
+    for (int k = 0; k < kND; ++k)
+      if (!SPLIT || z0 + k < z1) fill(z0 + k, k);
+    if (C::CORNER && lane >= z0 && lane < z1) {
       // pencil (M, M), plane `lane`
       const int z = lane;
       V ca, cb;
@@ -595,7 +613,7 @@ __device__ __forceinline__ void stage_block(const StagePtrs<T>& a, const StageCo
     }
     __syncwarp();
     int ds = kND - 1, dp = 0;
-    for (int z = kND; z <= M; ++z) {
+    for (int z = z0 + kND; z < z1; ++z) {
       // iteration z - 1 may start: every warp has put plane z - 1, so it has finished iteration z - 3,
       // whose slot is free
       mbar_wait(&full[ds], (unsigned)dp, err);
@@ -617,21 +635,41 @@ __device__ __forceinline__ void stage_block(const StagePtrs<T>& a, const StageCo
     __syncwarp();
     if ((tid & 31) == 0) mbar_arrive(&full[sl]);
   };
+  // The planes beyond the upper z face, needed from iteration M - 2 on (each thread its own pencil's),
+  // requested far enough ahead that nobody waits for them.
+  auto load_upper = [&]() {
+    const T* p;
+    int ls, fcs;
+    z_face(5, x, y, p, ls, fcs);
+#pragma unroll
+    for (int k = 0; k < 3; ++k) {
+      if (AI) {
+#pragma unroll
+        for (int q = 0; q < (int)(4 * sizeof(T) / 16); ++q)
+          cp_async_16(zup + k * 4 * SP + lq + q * (16 / (int)sizeof(T)), p + k * ls + q * (16 / (int)sizeof(T)));
+      } else {
+#pragma unroll
+        for (int f = 0; f < 4; ++f) cp_async_elem(zup + (k * 4 + f) * SP + lp, p + k * ls + (size_t)f * fcs);
+      }
+    }
+  };
   int ds = 0, dp = 0;                     // slot and phase of the iteration
   if (work) {
-    issue_halos(0);
-    issue_halos(1);
-    if (act) buf[0].put(ci, qa[3], qb[3]);
+    if (SPLIT && act && z0 >= M - 2) load_upper();
+    issue_halos(z0);
+    if (!SPLIT || z0 + 1 < z1) issue_halos(z0 + 1);
+    else cp_async_commit();
+    if (act) buf[z0 & 3].put(ci, qa[3], qb[3]);
     cp_async_wait_group<1>();
     publish(0);
   }
-  Plane<T, PW>* B = buf;                  // the plane of iteration z
+  Plane<T, PW>* B = buf + (z0 & 3);       // the plane of iteration z
 #pragma unroll 1
-  for (int zb = 0; zb <= M && work; zb += 7) {
+  for (int zb = z0; zb < z1 && work; zb += 7) {
 #pragma unroll
     for (int j = 0; j < 7; ++j) {
       const int z = zb + j;
-      if (z > M) break;
+      if (z >= z1) break;
       // ring entries of planes z - 3 .. z + 3
       auto QA = [&](int k) -> V& { return qa[(j + 3 + k) % 7]; };
       auto QB = [&](int k) -> V& { return qb[(j + 3 + k) % 7]; };
@@ -639,27 +677,10 @@ __device__ __forceinline__ void stage_block(const StagePtrs<T>& a, const StageCo
       const T* sg = stg + (size_t)ds * nst * SP;
       ds = ds == kND - 1 ? 0 : ds + 1;
       dp ^= ds == 0;
-      if (z == 1 && act) {
-        // the planes beyond the upper z face, needed from iteration M - 2 on (each thread its own
-        // pencil's): far enough ahead that nobody waits for them
-        const T* p;
-        int ls, fcs;
-        z_face(5, x, y, p, ls, fcs);
-#pragma unroll
-        for (int k = 0; k < 3; ++k) {
-          if (AI) {
-#pragma unroll
-            for (int q = 0; q < (int)(4 * sizeof(T) / 16); ++q)
-              cp_async_16(zup + k * 4 * SP + lq + q * (16 / (int)sizeof(T)), p + k * ls + q * (16 / (int)sizeof(T)));
-          } else {
-#pragma unroll
-            for (int f = 0; f < 4; ++f) cp_async_elem(zup + (k * 4 + f) * SP + lp, p + k * ls + (size_t)f * fcs);
-          }
-        }
-      }
-      if (z + 2 <= M) issue_halos(z + 2);
+      if (z == z0 + 1 && act && (!SPLIT || (z0 < M - 2 && z1 > M - 2))) load_upper();
+      if (z + 2 < z1) issue_halos(z + 2);
       else cp_async_commit();
-      if (z < M) {
+      if (z + 1 < z1) {
         if (act) buf[(z + 1) & 3].put(ci, QA(1), QB(1));
         cp_async_wait_group<1>();
         publish(ds);
@@ -728,11 +749,13 @@ __device__ __forceinline__ void stage_block(const StagePtrs<T>& a, const StageCo
   }
 }
 
-template <typename T, int BS, int STAGE, bool PM>
+template <typename T, int BS, int STAGE, bool PM, bool SPLIT>
 __global__ void __launch_bounds__(Cfg<T, BS>::NT + 32, Cfg<T, BS>::MINB)
-k_stage(const StageK<T> a, const TopoK tp, const PhysK ph, int* err) {
+k_stage(const StageK<T> a, const TopoK tp, const PhysK ph, int* err, int nz) {
   constexpr int NS = Cfg<T, BS>::NS;
-  stage_block<T, BS, STAGE, PM, false>(a.p, a.kc, tp, ph, err, blockIdx.x / NS, blockIdx.x % NS);
+  if (!SPLIT) nz = 1;
+  const int rank = blockIdx.x / (NS * nz), q = blockIdx.x % (NS * nz), zp = q / NS;
+  stage_block<T, BS, STAGE, PM, false, SPLIT>(a.p, a.kc, tp, ph, err, rank, q % NS, zp * BS / nz, (zp + 1) * BS / nz);
 }
 
 // Persistent form over several independent instances: the CTAs walk the work list of
@@ -745,7 +768,7 @@ k_stage_multi(const StageConst<T> kc, const PhysK ph, const StageInst<T>* desc, 
   for (int w = blockIdx.x; w < nwork; w += gridDim.x) {
     const int2 it = work[w];
     const StageInst<T> d = desc[it.x];
-    stage_block<T, BS, STAGE, true, true>(d.p, kc, d.tp, ph, err, it.y, 0);
+    stage_block<T, BS, STAGE, true, true, false>(d.p, kc, d.tp, ph, err, it.y, 0, 0, BS);
     __syncthreads();                   // the next block reuses the shared arrays
   }
 }
@@ -772,12 +795,50 @@ __global__ void k_rk_coefs(const unsigned long long* maxbits, RkK p, double* rk)
   rk[8] = dt / 3.0; rk[9] = dt / 6.0;
 }
 
+// Parts of a block along z, a CTA each.  A CTA costs its start (six extra planes to load and a chain
+// of dependent reads, about five planes' time in FP32, one in FP64 where a plane is long) plus its
+// planes; the parts are chosen so that the waves of CTAs over the chip cost least: a grid of a few
+// dozen blocks would leave most of the SMs idle with one CTA per block.  n: the blocks that run side by
+// side (instances of a batch on several streams together fill a chip that one of them would not: with
+// each split by its own count a batch of 12 instances took 11.1 ms instead of 9.9).  Measured, ms per launch with
+// one part and with this rule's: 64 blocks of 17^3 FP32 0.0192 and 0.0133, FP64 0.213 and 0.116; FP64
+// 1472 blocks 2.365 and 2.347.  A grid that fills the chip keeps one part, in a form of the kernel
+// whose plane range the compiler knows (the split form spills registers there: 4608 blocks 0.426
+// against 0.393, 32768 blocks 2.63 against 2.42).
+template <typename T, int BS>
+int z_parts(int64_t n) {
+  using C = Cfg<T, BS>;
+  const int64_t slots = (int64_t)C::MINB * sm_count(), start = sizeof(T) == 4 ? 5 : 1;
+  int best = 1;
+  int64_t cost = -1;
+  for (int nz = 1; nz <= BS / 2; ++nz) {
+    const int64_t c = (n * C::NS * nz + slots - 1) / slots * (start + (BS + nz - 1) / nz);
+    if (cost < 0 || c < cost) {
+      cost = c;
+      best = nz;
+    }
+  }
+  return best;
+}
+
+template <typename T, int BS, int STAGE, bool PM, bool SPLIT>
+void launch_parts(const StageK<T>& s, const TopoK& t, const PhysK& p, int* err, int nz, cudaStream_t st) {
+  static std::atomic<unsigned long long> opted{0};
+  smem_opt_in_stage(k_stage<T, BS, STAGE, PM, SPLIT>, stage_smem<T, BS, STAGE>(true), opted);
+  const size_t dyn = stage_smem<T, BS, STAGE>(p.mask != 0);
+  k_stage<T, BS, STAGE, PM, SPLIT>
+      <<<(unsigned)(t.n * Cfg<T, BS>::NS * nz), Cfg<T, BS>::NT + 32, dyn, st>>>(s, t, p, err, nz);
+}
 template <typename T, int BS, int STAGE, bool PM>
 void launch_one(const StageK<T>& s, const TopoK& t, const PhysK& p, int* err, cudaStream_t st) {
-  static std::atomic<unsigned long long> opted{0};
-  smem_opt_in_stage(k_stage<T, BS, STAGE, PM>, stage_smem<T, BS, STAGE>(true), opted);
-  const size_t dyn = stage_smem<T, BS, STAGE>(p.mask != 0);
-  k_stage<T, BS, STAGE, PM><<<(unsigned)(t.n * Cfg<T, BS>::NS), Cfg<T, BS>::NT + 32, dyn, st>>>(s, t, p, err);
+  const int nz = PM ? z_parts<T, BS>(std::max(t.n, s.side_by_side)) : 1;
+  if constexpr (PM) {
+    if (nz > 1) {
+      launch_parts<T, BS, STAGE, PM, true>(s, t, p, err, nz, st);
+      return;
+    }
+  }
+  launch_parts<T, BS, STAGE, PM, false>(s, t, p, err, 1, st);
 }
 
 template <typename T, int BS>
@@ -822,12 +883,12 @@ StageConst<T> stage_constants(const PhysK& p, double c_acc, double c_out, const 
 
 template <typename T>
 void launch_stage_multi(int stage, int Bs, const PhysK& p, const StageInst<T>* desc, const int2* work, int64_t nwork,
-                        int ctas, int* err, cudaStream_t st) {
+                        int* err, cudaStream_t st) {
   if (nwork <= 0 || Bs == 33) return;     // the persistent form takes whole blocks (Bs <= 17)
   const StageConst<T> kc = stage_constants<T>(p, 0.0, 0.0);
-  const int nb = (int)std::min<int64_t>(nwork, (int64_t)std::max(ctas, 1));
   auto go = [&](auto bs, auto sg) {
     constexpr int BS = decltype(bs)::value, SG = decltype(sg)::value;
+    const int nb = (int)std::min<int64_t>(nwork, (int64_t)Cfg<T, BS>::MINB * sm_count());
     static std::atomic<unsigned long long> opted{0};
     smem_opt_in_stage(k_stage_multi<T, BS, SG>, stage_smem<T, BS, SG>(true), opted);
     const size_t dyn = stage_smem<T, BS, SG>(p.mask != 0);
@@ -864,9 +925,9 @@ void launch_rk_coefs(const unsigned long long* maxbits, const RkK& p, double* rk
 
 template void launch_stage<float>(int, int, const StageK<float>&, const TopoK&, const PhysK&, int*, cudaStream_t);
 template void launch_stage<double>(int, int, const StageK<double>&, const TopoK&, const PhysK&, int*, cudaStream_t);
-template void launch_stage_multi<float>(int, int, const PhysK&, const StageInst<float>*, const int2*, int64_t, int,
+template void launch_stage_multi<float>(int, int, const PhysK&, const StageInst<float>*, const int2*, int64_t,
                                         int*, cudaStream_t);
-template void launch_stage_multi<double>(int, int, const PhysK&, const StageInst<double>*, const int2*, int64_t, int,
+template void launch_stage_multi<double>(int, int, const PhysK&, const StageInst<double>*, const int2*, int64_t,
                                          int*, cudaStream_t);
 
 }  // namespace acm

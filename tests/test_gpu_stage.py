@@ -61,3 +61,35 @@ def test_steps_match_oracle(A, prec, Bs, leaves, extras):
         S.rk4(1e-3)
     err = rel_linf(f.read_fields().astype(np.float64), block_order_fields(S))
     assert max(err) < TOL[prec], err
+
+
+@pytest.mark.parametrize("leaves", [ONE, PAIR, GRADED], ids=["one", "pair", "graded"])
+@pytest.mark.parametrize("Bs", [9, 17])
+def test_vjp_is_the_transpose_of_the_steps(A, Bs, leaves):
+    """<w, dF v> = <dF^T w, v> for two FP64 steps F with mask and sponge: dF v by central differences
+    of the steps, dF^T w by the vector-Jacobian product (kept stage states point-major; same-level,
+    finer and coarser faces).  The perturbation 1e-4 leaves a difference error of 1e-8 of the second
+    and third derivatives (order 1 here) and a rounding error of 1e-16 / 1e-4: 1e-6 of the norms
+    bounds both."""
+    f = A.Forest(_grid(leaves, Bs, 64), _phys(True))
+    f.set_leaves(leaves)
+    f.set_mask(A.ACM_MASK_SPHERE, (0.8, 0.5, 0.5, 0.2, 0.04))
+    fo = oracle_forest(_grid(leaves, Bs, 64), leaves=leaves, max_blocks=96)
+    S = oracle_solver(fo, _phys(True))
+    L = (1.0, 1.0, 1.0) if leaves == ONE else (2.0, 1.0, 1.0)
+
+    def field(seed):
+        fill_from_function(S, lambda X, Y, Z: smooth_field(X, Y, Z, L, seed))
+        return block_order_fields(S).copy()
+
+    U, v, w, e = field(5), field(6), field(7), 1e-4
+    out = []
+    for s in (1.0, -1.0):
+        f.write_fields(U + s * e * v)
+        for _ in range(2):
+            f.rk4_step(1e-3)
+        out.append(f.read_fields().copy())
+    f.write_fields(U)
+    g, _ = f.adjoint_vjp(2, 1e-3, w)
+    a, b = float((w * (out[0] - out[1])).sum() / (2 * e)), float((g * v).sum())
+    assert abs(a - b) <= 1e-6 * np.linalg.norm(w) * np.linalg.norm(v), (a, b)
