@@ -357,6 +357,36 @@ __global__ void __launch_bounds__(kNT) k_sync_ext(const T* reg, T* out, int g, c
 // component and the x-pass of the next share a phase (they touch different buffers).
 // Dynamic shared memory: c [4][NC^3], px [NC][NC][Bs], py [NC][Bs][Bs] in T, then the
 // neighbourhood.
+//
+// The block's indicator and mask range from the warps' partial results red[0..3] (largest detail of
+// each component), red[4], red[5] (least and largest chi), by the first warp: a lane per row, so that
+// the four FP64 divisions run at once (one thread doing them in turn held the GPU's few FP64 units for
+// a third of the kernel's time).
+template <typename T, int NT>
+__device__ __forceinline__ void block_indicator(int tid, const T (&red)[6][NT / 32], const unsigned long long* norm_bits,
+                                                bool mask, double* ind, double* chirange) {
+  if (tid >= 32) return;
+  T m = red[tid < 6 ? tid : 0][0];
+  for (int k = 1; k < NT / 32; ++k) {
+    const T t = red[tid < 6 ? tid : 0][k];
+    if (tid == 4 ? t < m : t > m) m = t;
+  }
+  // global max norm of component f, as left by the max-norm reduction (non-negative bits)
+  const double nf = __longlong_as_double((long long)norm_bits[tid & 3]);
+  const double inv = nf > 0.0 ? 1.0 / nf : 0.0;
+  const double r = inv == 0.0 ? 0.0 : (double)m * inv;
+  double best = 0.0;
+#pragma unroll
+  for (int f = 0; f < 4; ++f) {
+    const double rf = __shfl_sync(0xffffffffu, r, f);
+    best = rf > best ? rf : best;
+  }
+  const T mn = __shfl_sync(0xffffffffu, m, 4), mx = __shfl_sync(0xffffffffu, m, 5);
+  if (tid == 0) {
+    *ind = best;
+    *chirange = mask ? (double)mx - (double)mn : 0.0;
+  }
+}
 template <typename T, int BS>
 struct DetSmem {
   static constexpr int NT = ((BS * BS + 31) / 32) * 32;
@@ -442,7 +472,6 @@ __global__ void __launch_bounds__(DetSmem<T, BS>::NT) k_details(const T* reg, co
       for (int i = 0; i < BS; ++i) px[tid * BS + i] = dd4_line<T, BS>(cv, i);
     }
   };
-  double best = 0.0;
   T u[BS];
   xpass(0);
   for (int f = 0; f < 4; ++f) {
@@ -486,25 +515,7 @@ __global__ void __launch_bounds__(DetSmem<T, BS>::NT) k_details(const T* reg, co
   }
   if (lane == 0) { red[4][wid] = tmin; red[5][wid] = tmax; }
   __syncthreads();
-  if (tid == 0) {
-    for (int f = 0; f < 4; ++f) {
-      // global max norm of component f, as left by the max-norm reduction (non-negative bits)
-      const double nf = __longlong_as_double((long long)norm_bits[f]);
-      const double inv = nf > 0.0 ? 1.0 / nf : 0.0;
-      if (inv == 0.0) continue;
-      T m = red[f][0];
-      for (int k = 1; k < NT / 32; ++k) m = red[f][k] > m ? red[f][k] : m;
-      const double r = (double)m * inv;
-      best = r > best ? r : best;
-    }
-    T mn = red[4][0], mx = red[5][0];
-    for (int k = 1; k < NT / 32; ++k) {
-      mn = red[4][k] < mn ? red[4][k] : mn;
-      mx = red[5][k] > mx ? red[5][k] : mx;
-    }
-    ind[rank] = best;
-    chirange[rank] = chi ? (double)mx - (double)mn : 0.0;
-  }
+  block_indicator<T, NT>(tid, red, norm_bits, chi != nullptr, ind + rank, chirange + rank);
 }
 
 // Block indicators of Bs = 33 blocks: the same passes with one component's coarse samples in
@@ -614,41 +625,22 @@ k_details_big(const T* reg, const T* chi, const int32_t* blist, const int32_t* r
   }
   if (lane == 0) { red[4][wid] = tmin; red[5][wid] = tmax; }
   __syncthreads();
-  if (tid == 0) {
-    double best = 0.0;
-    for (int f = 0; f < 4; ++f) {
-      const double nf = __longlong_as_double((long long)norm_bits[f]);
-      const double inv = nf > 0.0 ? 1.0 / nf : 0.0;
-      if (inv == 0.0) continue;
-      T m = red[f][0];
-      for (int k = 1; k < NT / 32; ++k) m = red[f][k] > m ? red[f][k] : m;
-      const double r = (double)m * inv;
-      best = r > best ? r : best;
-    }
-    T mn = red[4][0], mx = red[5][0];
-    for (int k = 1; k < NT / 32; ++k) {
-      mn = red[4][k] < mn ? red[4][k] : mn;
-      mx = red[5][k] > mx ? red[5][k] : mx;
-    }
-    ind[rank] = best;
-    chirange[rank] = chi ? (double)mx - (double)mn : 0.0;
-  }
+  block_indicator<T, NT>(tid, red, norm_bits, chi != nullptr, ind + rank, chirange + rank);
 }
 
 // ---- (5) max norms (Sec. 2.3 u_max, Sec. 3.4 normalisation) ------------------------------------
 template <typename T, int BS>
-__global__ void __launch_bounds__(kNT) k_maxnorm(const T* reg, const int32_t* blist, unsigned long long* out) {
+__global__ void __launch_bounds__(kNT) k_maxnorm(const T* reg, const int32_t* blist, unsigned long long* out, int parts) {
   using L = Lay<T, BS>;
-  const int slot = blist[blockIdx.x];
+  const int slot = blist[blockIdx.x / parts];
   const T* b = reg + (size_t)slot * L::BLK;
   // arithmetic in the field precision (an FP32 field gives an FP32 norm, stored as double);
   // m[4] holds the squared magnitude, its root is taken once at the end.  The maxima propagate
   // NaN (a comparison with NaN is false, so a plain maximum would drop it): a non-finite state
   // reaches the host as a non-finite norm.
   T m[5] = {T(0), T(0), T(0), T(0), T(0)};
-  auto keep = [](T a, T m) { return (a > m || a != a) ? a : m; };
   constexpr int N = BS * BS * BS, U = 4;
-  for (int base = threadIdx.x; base < N; base += kNT * U) {
+  for (int base = (blockIdx.x % parts) * kNT * U + threadIdx.x; base < N; base += parts * kNT * U) {
     T v[U][4];
 #pragma unroll
     for (int k = 0; k < U; ++k) {
@@ -661,22 +653,22 @@ __global__ void __launch_bounds__(kNT) k_maxnorm(const T* reg, const int32_t* bl
     for (int k = 0; k < U; ++k) {
 #pragma unroll
       for (int f = 0; f < 4; ++f) {
-        m[f] = keep(tabs(v[k][f]), m[f]);
+        m[f] = max_magnitude(v[k][f], m[f]);
       }
-      m[4] = keep(mag2(v[k][0], v[k][1], v[k][2]), m[4]);
+      m[4] = max_magnitude(mag2(v[k][0], v[k][1], v[k][2]), m[4]);
     }
   }
   __shared__ T red[5][kNT / 32];
 #pragma unroll
   for (int k = 0; k < 5; ++k) {
     T mk = m[k];
-    for (int o = 16; o > 0; o >>= 1) mk = keep(__shfl_xor_sync(0xffffffffu, mk, o), mk);
+    for (int o = 16; o > 0; o >>= 1) mk = max_magnitude(__shfl_xor_sync(0xffffffffu, mk, o), mk);
     if ((threadIdx.x & 31) == 0) red[k][threadIdx.x >> 5] = mk;
   }
   __syncthreads();
   if (threadIdx.x < 5) {
     T mk = T(0);
-    for (int w = 0; w < kNT / 32; ++w) mk = keep(red[threadIdx.x][w], mk);
+    for (int w = 0; w < kNT / 32; ++w) mk = max_magnitude(red[threadIdx.x][w], mk);
     const double d = threadIdx.x == 4 ? (double)tsqrt(mk) : (double)mk;
     atomicMax(out + threadIdx.x, (unsigned long long)__double_as_longlong(d));
   }
@@ -1395,62 +1387,87 @@ __global__ void __launch_bounds__(kNT) k_ic(T* reg, const int32_t* blist, const 
   }
 }
 
-// chi along the z-column (ix, iy) of one block (out: the block's mask component).
-template <typename T, int BS>
-__device__ __forceinline__ void mask_column(T* out, const int ix, const int iy, const int uniform, const int4 bi,
-                                            const PhysK& ph, const MaskK& m, const double h) {
+// The mask's constants in the field precision, rounded once on the host (FP64 conversions are as
+// slow as FP64 arithmetic on this GPU: 19 of them in every thread cost more than the column's own
+// work), and in float for the estimates below.  tol bounds the error of a distance computed in float
+// from float coordinates: 64 roundings of the largest coordinate difference that occurs.
+template <typename T>
+struct MaskC {
+  T p[19];
+  float pf[19];
+  float far, tol;                // the distance beyond which chi is exactly 0 or 1, and that bound
+  T h[kMaxLevel + 1];
+  float hf[kMaxLevel + 1];
+};
+template <typename T>
+inline MaskC<T> mask_constants(const MaskK& m, const PhysK& ph) {
+  MaskC<T> c;
+  for (int k = 0; k < 19; ++k) {
+    c.p[k] = T(m.p[k]);
+    c.pf[k] = (float)m.p[k];
+  }
+  for (int J = 0; J <= kMaxLevel; ++J) {
+    c.h[J] = T(ph.h[J]);
+    c.hf[J] = (float)ph.h[J];
+  }
+  double E = 0.0;
+  for (int a = 0; a < 3; ++a) {
+    E += ph.nroot[a] * ph.root_len;
+    E += m.kind == 2 ? fabs(m.p[9 + a]) + fabs(m.p[12 + a]) + fabs(m.p[15 + a]) : fabs(m.p[a]);
+  }
+  if (m.kind == 1) E += fabs(m.p[3]);
+  c.far = (float)((sizeof(T) == 4 ? 10.0 : 20.0) * 1.05 * (m.kind == 2 ? m.p[18] : m.p[4]));
+  c.tol = (float)(64.0 * 6e-8 * E);
+  return c;
+}
+// The signed distance of the offset r from the sphere's centre or the box's pivot.
+template <typename T>
+__device__ __forceinline__ T sphere_distance(const T* p, T rx, T ry, T rz) {
+  return tsqrt(rx * rx + ry * ry + rz * rz) - p[3];
+}
+template <typename T>
+__device__ __forceinline__ T box_distance(const T* p, T rx, T ry, T rz) {
+  T out2 = T(0), qmax = T(-1e30);
+#pragma unroll
+  for (int k = 0; k < 3; ++k) {
+    const T xb = p[k] * rx + p[3 + k] * ry + p[6 + k] * rz;     // (R^T r)_k
+    const T q = (xb - p[12 + k] < T(0) ? p[12 + k] - xb : xb - p[12 + k]) - p[15 + k];
+    if (q > T(0)) out2 += q * q;
+    qmax = q > qmax ? q : qmax;
+  }
+  return tsqrt(out2) + (qmax < T(0) ? qmax : T(0));
+}
+
+// chi along the z-column (ix, iy) of one block (out: the block's mask component), evaluated in the
+// field precision.  FP64 fields: points that a float estimate of the distance places beyond 20 delta
+// take 0 or 1, their exact value, without the FP64 root and tanh.
+template <typename T, int BS, int KIND>
+__device__ __forceinline__ void mask_column(T* out, const int ix, const int iy, const int4 bi, const PhysK& ph,
+                                            const MaskC<T>& m) {
   using L = Lay<T, BS>;
   constexpr int M = L::M;
-  if (uniform >= 0) {
-#pragma unroll
-    for (int iz = 0; iz < BS; ++iz) out[L::idx(ix, iy, iz)] = T(uniform);
-    return;
-  }
-  if (m.kind == 2) {
-    // signed distance to the box in the body frame, in the field precision
-    const T hT = T(h);
-    T Rm[9], x0[3], cb[3], hb[3];
-    for (int k = 0; k < 9; ++k) Rm[k] = T(m.p[k]);
-    for (int a = 0; a < 3; ++a) {
-      x0[a] = T(m.p[9 + a]);
-      cb[a] = T(m.p[12 + a]);
-      hb[a] = T(m.p[15 + a]);
-    }
-    const T dl = T(m.p[18]);
-    const T cut = T(sizeof(T) == 4 ? 10.0 : 20.0) * dl;
-    const T rx = T(lattice(ph, bi, 0, ix, M)) * hT - x0[0], ry = T(lattice(ph, bi, 1, iy, M)) * hT - x0[1];
-    for (int iz = 0; iz < BS; ++iz) {
-      const T rz = T(lattice(ph, bi, 2, iz, M)) * hT - x0[2];
-      T out2 = T(0), qmax = T(-1e30);
-      for (int k = 0; k < 3; ++k) {
-        const T xb = Rm[k] * rx + Rm[3 + k] * ry + Rm[6 + k] * rz;     // (R^T r)_k
-        const T q = (xb - cb[k] < T(0) ? cb[k] - xb : xb - cb[k]) - hb[k];
-        if (q > T(0)) out2 += q * q;
-        qmax = q > qmax ? q : qmax;
-      }
-      const T d = tsqrt(out2) + (qmax < T(0) ? qmax : T(0));
-      T c;
-      if (d > cut) c = T(0);
-      else if (d < -cut) c = T(1);
-      else c = T(0.5) * (T(1) - ttanh(d / dl));
-      out[L::idx(ix, iy, iz)] = c;
-    }
-    return;
-  }
-  // evaluated in the field precision: FP64 fields in double, FP32 fields in float; the
-  // conversions of the constants are done once, outside the point loop
-  const T hT = T(h);
-  const T c0 = T(m.p[0]), c1 = T(m.p[1]), c2 = T(m.p[2]), R = T(m.p[3]), dl = T(m.p[4]);
+  constexpr int O = KIND == 2 ? 9 : 0;                 // the pivot's or centre's place in the parameters
+  const T hT = m.h[bi.x], dl = m.p[KIND == 2 ? 18 : 4];
+  const float hf = m.hf[bi.x];
   // beyond 10 delta (FP32) / 20 delta (FP64) tanh(d/delta) rounds to exactly +-1
   const T cut = T(sizeof(T) == 4 ? 10.0 : 20.0) * dl;
   // coordinates i h with i the wrapped lattice index (exact when h is dyadic, as for
   // power-of-two root sides)
-  const T dx = T(lattice(ph, bi, 0, ix, M)) * hT - c0, dy = T(lattice(ph, bi, 1, iy, M)) * hT - c1;
-#pragma unroll
+  const T rx = T(lattice(ph, bi, 0, ix, M)) * hT - m.p[O], ry = T(lattice(ph, bi, 1, iy, M)) * hT - m.p[O + 1];
+#pragma unroll KIND == 2 ? 1 : BS
   for (int iz = 0; iz < BS; ++iz) {
-    const T dz = T(lattice(ph, bi, 2, iz, M)) * hT - c2;
-    const T d = tsqrt(dx * dx + dy * dy + dz * dz) - R;
     T c;
+    if constexpr (sizeof(T) == 8) {
+      const float rzf = (float)lattice(ph, bi, 2, iz, M) * hf - m.pf[O + 2];
+      const float df = KIND == 2 ? box_distance<float>(m.pf, (float)rx, (float)ry, rzf)
+                                 : sphere_distance<float>(m.pf, (float)rx, (float)ry, rzf);
+      if (fabsf(df) > m.far + m.tol) {
+        out[L::idx(ix, iy, iz)] = df > 0.f ? T(0) : T(1);
+        continue;
+      }
+    }
+    const T rz = T(lattice(ph, bi, 2, iz, M)) * hT - m.p[O + 2];
+    const T d = KIND == 2 ? box_distance<T>(m.p, rx, ry, rz) : sphere_distance<T>(m.p, rx, ry, rz);
     if (d > cut) c = T(0);
     else if (d < -cut) c = T(1);
     else c = T(0.5) * (T(1) - ttanh(d / dl));
@@ -1460,61 +1477,51 @@ __device__ __forceinline__ void mask_column(T* out, const int ix, const int iy, 
 
 template <typename T, int BS>
 __global__ void __launch_bounds__(ColCfg<BS>::NT) k_mask(T* chi, const int32_t* blist, const int32_t* ranks,
-                                                         const int4* binfo, const PhysK ph, const MaskK m) {
+                                                         const int4* binfo, const PhysK ph, const int kind,
+                                                         const MaskC<T> m) {
   using L = Lay<T, BS>;
   constexpr int M = L::M;
   const int rank = ranks ? ranks[blockIdx.x] : (int)blockIdx.x;
   const int slot = blist[rank];
   const int4 bi = binfo[rank];
-  const double h = ph.h[bi.x];
-  // A block that lies entirely farther than 40 delta from the sphere surface has tanh(d/delta)
-  // = +-1 exactly in double precision at all its points (1 - tanh(40) < 1e-34): chi is exactly
-  // 0 or 1 there and needs no transcendental.  Blocks on the periodic seam are evaluated fully.
-  // One thread decides (FP64), the block reads the answer.
-  __shared__ int s_uniform;
-  if (threadIdx.x == 0) {
-    int uniform = 0;
-    if (m.kind == 1) {
-      uniform = -1;
-      const double lo[3] = {(double)bi.y * M * h, (double)bi.z * M * h, (double)bi.w * M * h};
-      const double L[3] = {ph.nroot[0] * ph.root_len, ph.nroot[1] * ph.root_len, ph.nroot[2] * ph.root_len};
-      bool seam = false;
-      double dmin2 = 0.0, dmax2 = 0.0;
-      for (int a = 0; a < 3; ++a) {
-        const double hi = lo[a] + M * h;
-        if (hi >= L[a]) seam = true;
-        const double c = m.p[a];
-        const double near = c < lo[a] ? lo[a] - c : (c > hi ? c - hi : 0.0);
-        const double far = fmax(fabs(c - lo[a]), fabs(hi - c));
-        dmin2 += near * near;
-        dmax2 += far * far;
-      }
-      if (!seam) {
-        if (sqrt(dmin2) - m.p[3] > 40.0 * m.p[4]) uniform = 0;
-        else if (sqrt(dmax2) - m.p[3] < -40.0 * m.p[4]) uniform = 1;
-      }
-    } else if (m.kind == 2) {
-      // rigid box: outside the sphere of radius p[22] around the pivot by more than 40 delta
-      uniform = -1;
-      const double lo[3] = {(double)bi.y * M * h, (double)bi.z * M * h, (double)bi.w * M * h};
-      const double L[3] = {ph.nroot[0] * ph.root_len, ph.nroot[1] * ph.root_len, ph.nroot[2] * ph.root_len};
-      bool seam = false;
-      double dmin2 = 0.0;
-      for (int a = 0; a < 3; ++a) {
-        const double hi = lo[a] + M * h;
-        if (hi >= L[a]) seam = true;
-        const double c = m.p[9 + a];
-        const double near = c < lo[a] ? lo[a] - c : (c > hi ? c - hi : 0.0);
-        dmin2 += near * near;
-      }
-      if (!seam && sqrt(dmin2) - m.p[22] > 40.0 * m.p[18]) uniform = 0;
+  // A block whose points all lie beyond 10 delta (FP32) / 20 delta (FP64) from the surface has chi
+  // exactly 0 or 1 everywhere and needs no transcendental: the distance is 1-Lipschitz, so its value at
+  // the block's centre, less the half diagonal, decides.  In float (its error bound added), by every
+  // thread (one thread's answer through shared memory took longer).  Blocks on the periodic seam are
+  // evaluated fully.
+  int uniform = 0;
+  if (kind == 1 || kind == 2) {
+    uniform = -1;
+    const float hf = m.hf[bi.x];
+    bool seam = false;
+    float r[3];
+    const int g[3] = {bi.y, bi.z, bi.w};
+    const int O = kind == 2 ? 9 : 0;
+#pragma unroll
+    for (int a = 0; a < 3; ++a) {
+      seam |= (long long)g[a] + 1 >= ((long long)ph.nroot[a] << bi.x);
+      r[a] = ((float)g[a] * M + 0.5f * M) * hf - (O ? m.pf[9 + a] : m.pf[a]);
     }
-    s_uniform = uniform;
+    if (!seam) {
+      const float d = kind == 2 ? box_distance<float>(m.pf, r[0], r[1], r[2])
+                                : sphere_distance<float>(m.pf, r[0], r[1], r[2]);
+      if (fabsf(d) - 0.8661f * M * hf > m.far + m.tol) uniform = d > 0.f ? 0 : 1;
+    }
   }
-  __syncthreads();
-  const int uniform = s_uniform;
-  for (int col = threadIdx.x; col < BS * BS; col += ColCfg<BS>::NT)
-    mask_column<T, BS>(chi + (size_t)slot * L::FS, col % BS, col / BS, uniform, bi, ph, m, h);
+  T* out = chi + (size_t)slot * L::FS;
+  if (uniform >= 0) {
+    // whole 16-byte words (the planes' padding included: nothing reads it)
+    union { T t[16 / sizeof(T)]; int4 v; } one;
+#pragma unroll
+    for (int k = 0; k < 16 / (int)sizeof(T); ++k) one.t[k] = T(uniform);
+    for (int i = threadIdx.x; i < BS * L::PP * (int)sizeof(T) / 16; i += ColCfg<BS>::NT)
+      reinterpret_cast<int4*>(out)[i] = one.v;
+    return;
+  }
+  for (int col = threadIdx.x; col < BS * BS; col += ColCfg<BS>::NT) {
+    if (kind == 2) mask_column<T, BS, 2>(out, col % BS, col / BS, bi, ph, m);
+    else mask_column<T, BS, 1>(out, col % BS, col / BS, bi, ph, m);
+  }
 }
 
 // ---- (9) diagnostics: raw per-block sums over the half-open points [0, M-1]^3 -----------------
@@ -1608,27 +1615,49 @@ __global__ void __launch_bounds__(1024) k_diag_sum(const double* part, const int
 }
 
 // ---- (10) dense <-> pool ---------------------------------------------------------------------------
+// A CTA per (block, component), eight words in flight per thread: a CTA per block with one word at a
+// time took 38 us on 64 blocks of 17^3 as on 576.
 template <typename T, int BS>
 __global__ void __launch_bounds__(kNT) k_gather(const T* reg, T* dense, const int32_t* blist, int ncomp, int comp_stride_blk) {
   using L = Lay<T, BS>;
-  const int slot = blist[blockIdx.x];
-  const int n = ncomp * BS * BS * BS;
-  for (int i = threadIdx.x; i < n; i += kNT) {
-    const int f = i / (BS * BS * BS), r = i % (BS * BS * BS);
-    const int x = r % BS, y = (r / BS) % BS, z = r / (BS * BS);
-    dense[(size_t)blockIdx.x * n + i] = reg[(size_t)slot * comp_stride_blk + (size_t)f * L::FS + L::idx(x, y, z)];
+  constexpr int N3 = BS * BS * BS, PAD = L::PP - BS * BS;
+  const int f = blockIdx.x % ncomp;
+  const T* s = reg + (size_t)blist[blockIdx.x / ncomp] * comp_stride_blk + (size_t)f * L::FS;
+  T* d = dense + (size_t)blockIdx.x * N3;
+  for (int i = threadIdx.x; i < N3; i += 8 * kNT) {
+    T v[8];
+#pragma unroll
+    for (int u = 0; u < 8; ++u) {
+      const int j = i + u * kNT;
+      if (j < N3) v[u] = s[j + j / (BS * BS) * PAD];
+    }
+#pragma unroll
+    for (int u = 0; u < 8; ++u) {
+      const int j = i + u * kNT;
+      if (j < N3) d[j] = v[u];
+    }
   }
 }
 
 template <typename T, int BS>
 __global__ void __launch_bounds__(kNT) k_scatter(const T* dense, T* reg, const int32_t* blist, int ncomp, int comp_stride_blk) {
   using L = Lay<T, BS>;
-  const int slot = blist[blockIdx.x];
-  const int n = ncomp * BS * BS * BS;
-  for (int i = threadIdx.x; i < n; i += kNT) {
-    const int f = i / (BS * BS * BS), r = i % (BS * BS * BS);
-    const int x = r % BS, y = (r / BS) % BS, z = r / (BS * BS);
-    reg[(size_t)slot * comp_stride_blk + (size_t)f * L::FS + L::idx(x, y, z)] = dense[(size_t)blockIdx.x * n + i];
+  constexpr int N3 = BS * BS * BS, PAD = L::PP - BS * BS;
+  const int f = blockIdx.x % ncomp;
+  T* o = reg + (size_t)blist[blockIdx.x / ncomp] * comp_stride_blk + (size_t)f * L::FS;
+  const T* d = dense + (size_t)blockIdx.x * N3;
+  for (int i = threadIdx.x; i < N3; i += 8 * kNT) {
+    T v[8];
+#pragma unroll
+    for (int u = 0; u < 8; ++u) {
+      const int j = i + u * kNT;
+      if (j < N3) v[u] = d[j];
+    }
+#pragma unroll
+    for (int u = 0; u < 8; ++u) {
+      const int j = i + u * kNT;
+      if (j < N3) o[j + j / (BS * BS) * PAD] = v[u];
+    }
   }
 }
 
@@ -1744,7 +1773,9 @@ void launch_details(int Bs, const T* reg, const T* chi, const int32_t* blist, co
 template <typename T>
 void launch_maxnorm(int Bs, const T* reg, const int32_t* blist, int64_t n, unsigned long long* out, cudaStream_t st) {
   if (n <= 0) return;
-  ACM_BS_DISPATCH(Bs, k_maxnorm, <<<grid1(n), kNT, 0, st>>>(reg, blist, out));
+  // a grid of fewer blocks than the chip holds CTAs (eight per SM) splits each over four
+  const int parts = n < 8 * sm_count() ? 4 : 1;
+  ACM_BS_DISPATCH(Bs, k_maxnorm, <<<grid1(n * parts), kNT, 0, st>>>(reg, blist, out, parts));
 }
 template <typename T, int BS>
 void launch_refine_bs(const T* src, T* dst, const int32_t* tasks, int64_t n, const int32_t* blist,
@@ -1808,12 +1839,13 @@ template <typename T>
 void launch_mask(int Bs, T* chi, const int32_t* blist, const int32_t* ranks, int64_t n, const int4* binfo,
                  const PhysK& p, const MaskK& m, cudaStream_t st) {
   if (n <= 0) return;
+  const MaskC<T> c = mask_constants<T>(m, p);
   if (Bs == 33) {
-    if constexpr (sizeof(T) == 4) k_mask<T, 33><<<grid1(n), ColCfg<33>::NT, 0, st>>>(chi, blist, ranks, binfo, p, m);
+    if constexpr (sizeof(T) == 4) k_mask<T, 33><<<grid1(n), ColCfg<33>::NT, 0, st>>>(chi, blist, ranks, binfo, p, m.kind, c);
   } else if (Bs == 17) {
-    k_mask<T, 17><<<grid1(n), ColCfg<17>::NT, 0, st>>>(chi, blist, ranks, binfo, p, m);
+    k_mask<T, 17><<<grid1(n), ColCfg<17>::NT, 0, st>>>(chi, blist, ranks, binfo, p, m.kind, c);
   } else {
-    k_mask<T, 9><<<grid1(n), ColCfg<9>::NT, 0, st>>>(chi, blist, ranks, binfo, p, m);
+    k_mask<T, 9><<<grid1(n), ColCfg<9>::NT, 0, st>>>(chi, blist, ranks, binfo, p, m.kind, c);
   }
 }
 template <typename T>
@@ -1836,7 +1868,7 @@ void launch_gather(int Bs, const T* reg, T* dense, const int32_t* blist, int64_t
   if (n <= 0) return;
   const int stride = (int)layout_info(sizeof(T) == 8 ? 64 : 32, Bs).BLK;
   const int cstride = ncomp == 1 ? (int)layout_info(sizeof(T) == 8 ? 64 : 32, Bs).FS : stride;
-  ACM_BS_DISPATCH(Bs, k_gather, <<<grid1(n), kNT, 0, st>>>(reg, dense, blist, ncomp, cstride));
+  ACM_BS_DISPATCH(Bs, k_gather, <<<grid1(n * ncomp), kNT, 0, st>>>(reg, dense, blist, ncomp, cstride));
 }
 template <typename T>
 void launch_scatter(int Bs, const T* dense, T* reg, const int32_t* blist, int64_t n, int ncomp, cudaStream_t st) {
@@ -1844,7 +1876,7 @@ void launch_scatter(int Bs, const T* dense, T* reg, const int32_t* blist, int64_
   // a one-component register (the mask) has one component per slot, like launch_gather's
   const int stride = (int)layout_info(sizeof(T) == 8 ? 64 : 32, Bs).BLK;
   const int cstride = ncomp == 1 ? (int)layout_info(sizeof(T) == 8 ? 64 : 32, Bs).FS : stride;
-  ACM_BS_DISPATCH(Bs, k_scatter, <<<grid1(n), kNT, 0, st>>>(dense, reg, blist, ncomp, cstride));
+  ACM_BS_DISPATCH(Bs, k_scatter, <<<grid1(n * ncomp), kNT, 0, st>>>(dense, reg, blist, ncomp, cstride));
 }
 
 #define ACM_INST(T)                                                                                        \

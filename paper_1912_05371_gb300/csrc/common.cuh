@@ -135,6 +135,27 @@ __device__ __forceinline__ T mag2(T u, T v, T w) {
   return fma(w, w, s);
 }
 
+// max(|a|, m) for a non-negative m; a NaN a is dropped.  FP64 magnitudes are compared as their bit
+// patterns (the same order) on the integer units instead of the GPU's few FP64 ones.
+__device__ __forceinline__ float max_number(float a, float m) {
+  a = fabsf(a);
+  return a > m ? a : m;
+}
+__device__ __forceinline__ double max_number(double a, double m) {
+  const long long x = __double_as_longlong(a) & 0x7fffffffffffffffll, y = __double_as_longlong(m);
+  return __longlong_as_double(x > y && x <= 0x7ff0000000000000ll ? x : y);
+}
+// max(|a|, m) for a non-negative m, propagating NaN (a comparison with NaN is false, so a plain
+// maximum would drop it; as bit patterns a NaN is above everything).
+__device__ __forceinline__ float max_magnitude(float a, float m) {
+  a = fabsf(a);
+  return (a > m || a != a) ? a : m;
+}
+__device__ __forceinline__ double max_magnitude(double a, double m) {
+  const long long x = __double_as_longlong(a) & 0x7fffffffffffffffll, y = __double_as_longlong(m);
+  return __longlong_as_double(x > y ? x : y);
+}
+
 // DD-4 prediction of one line (Sec. 3.1): from NC = M/2 + 3 coarse samples c[k] at coarse
 // index k - 1 (fine index 2k - 2), the fine value at fine index i = 0..M: the sample itself at
 // even i, the 4-point stencil (-1, 9, 9, -1)/16 around it at odd i.  The sum runs left to right.

@@ -76,6 +76,7 @@ struct StageConst {
   T om[3], x0[3];
   T ih[kMaxLevel + 1];      // a_1 / h_J
   T ih2[kMaxLevel + 1];     // 1 / (12 h_J^2)
+  T h[kMaxLevel + 1];
 };
 
 struct MaskK;

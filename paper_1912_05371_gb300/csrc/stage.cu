@@ -492,7 +492,7 @@ __device__ __forceinline__ void stage_block(const StagePtrs<T>& a, const StageCo
   };
   // solid velocity of a moving body at lattice point (i, j, k): omega x (x - x_0)
   auto solid = [&](int i, int j, int k, T (&us)[3]) {
-    const T hT = T(ph.h[bi.x]);
+    const T hT = kc.h[bi.x];
     const T rx = T(lattice_index(ph, bi, 0, i, M)) * hT - kc.x0[0];
     const T ry = T(lattice_index(ph, bi, 1, j, M)) * hT - kc.x0[1];
     const T rz = T(lattice_index(ph, bi, 2, k, M)) * hT - kc.x0[2];
@@ -531,12 +531,8 @@ __device__ __forceinline__ void stage_block(const StagePtrs<T>& a, const StageCo
   T nm[5] = {T(0), T(0), T(0), T(0), T(0)};   // stage 4: max |u|,|v|,|w|,|p|, |(u,v,w)|^2
   auto norms_of = [&](const T (&nv)[4]) {
 #pragma unroll
-    for (int f = 0; f < 4; ++f) {
-      const T av = nv[f] < T(0) ? -nv[f] : nv[f];
-      nm[f] = av > nm[f] ? av : nm[f];
-    }
-    const T m2 = mag2(nv[0], nv[1], nv[2]);
-    nm[4] = m2 > nm[4] ? m2 : nm[4];
+    for (int f = 0; f < 4; ++f) nm[f] = max_number(nv[f], nm[f]);
+    nm[4] = max_number(mag2(nv[0], nv[1], nv[2]), nm[4]);
   };
   const int nst = staged_arrays<STAGE>(ph.mask != 0);
   // this CTA's rows of a plane, widened to 16-byte boundaries inside the padded plane
@@ -875,6 +871,7 @@ StageConst<T> stage_constants(const PhysK& p, double c_acc, double c_out, const 
   for (int J = 0; J <= kMaxLevel; ++J) {
     c.ih[J] = T(p.a1 / p.h[J]);
     c.ih2[J] = T(1.0 / (12.0 * p.h[J] * p.h[J]));
+    c.h[J] = T(p.h[J]);
   }
   return c;
 }
