@@ -9,15 +9,13 @@
 // face halos (3 layers) from the finest leaf holding a point, else by the tensor DD-4 prediction
 // (Sec. 3.1, 4.2), and loc is the block-local stencil arithmetic.  The adjoint of one stage,
 // nu = W^T E^T loc^T kappa with kappa = c_lam lam + c_nu nu' (the RK4 adjoint combination), takes
-// four launches:
+// three launches, four with a moving body:
 //   k_adj_stage      loc^T at every block's own interior points, in gather form (a z-march like
 //                    the forward stage kernel), with the combination for kappa, the running sum
 //                    of the stage nus and the mask sensitivity fused in;
-//   k_adj_samelevel  E^T of the face-halo targets that same-level neighbours read from a block,
-//                    gathered by that block (no atomics);
-//   k_adj_halo       loc^T at the face-halo points toward finer and coarser faces and E^T: added
-//                    to the points they were read from (the finest leaf holding the point, or its
-//                    DD-4 prediction's even points);
+//   k_adj_body       the moving body's parameter sensitivity (a moving body only);
+//   k_adj_halo       loc^T at the face-halo points and E^T: added to the points they were read from
+//                    (the finest leaf holding the point, or its DD-4 prediction's even points);
 //   k_adj_fw_T       W^T: a boundary point held by a finer leaf passes its value to that leaf's
 //                    point and is cleared.
 // The objective's direct terms and the reduction of the mask sensitivity onto the sphere's centre
@@ -40,6 +38,7 @@ constexpr int kNA = 256;
 
 // faces: 0 -x, 1 +x, 2 -y, 3 +y, 4 -z, 5 +z ; box index of the face neighbour
 __constant__ int kFaceBox[6] = {12, 14, 10, 16, 4, 22};
+
 
 __device__ __forceinline__ double lattice_coord(const PhysK& ph, int4 bi, int a, int i, int M, double h) {
   const int g = a == 0 ? bi.y : (a == 1 ? bi.z : bi.w);
@@ -76,29 +75,55 @@ __device__ __forceinline__ BoxPoint box_point(const MaskK& m, double rx, double 
     if (q[k] > 0.0) n2 += q[k] * q[k];
     if (q[k] > qmax) { qmax = q[k]; kmax = k; }
   }
-  const double nout = sqrt(n2);
-  double gd = 0.0;                                     // grad d . d x_b / dtheta
-  if (nout > 0.0) {
+  // d chi/dtheta = -sech^2(d/delta) / (2 delta) grad d . d x_b/dtheta, sech^2 t = 4 e / (1 + e)^2 with
+  // e = exp(-2 |t|); one division for all of it
+  double gd = 0.0, nout = 0.0, den = 1.0;
+  if (n2 > 0.0) {
+    nout = sqrt(n2);
+    den = nout;
     for (int k = 0; k < 3; ++k)
-      if (q[k] > 0.0) gd += q[k] / nout * sg[k] * dxb[k];
+      if (q[k] > 0.0) gd += q[k] * sg[k] * dxb[k];
   } else {
     gd = sg[kmax] * dxb[kmax];
   }
   const double d = nout + (qmax < 0.0 ? qmax : 0.0);
-  const double th = tanh(d / m.p[18]);
-  o.dchi = -0.5 / m.p[18] * (1.0 - th * th) * gd;
+  const double e = exp(-2.0 * fabs(d) * m.p[36]);
+  o.dchi = -2.0 * m.p[36] * e * gd / ((1.0 + e) * (1.0 + e) * den);
   return o;
 }
 
 // A float estimate of the box's signed distance at offset r (the distance part of box_point, in
-// float): it decides which points are so far from the surface that tanh(d/delta) is +-1 in the
-// field precision (exactly in FP64 beyond 19.1 delta), where d chi/dtheta vanishes and chi is 0
-// (outside) or 1 (inside), and the FP64 distance and tanh need not be evaluated.
-__device__ __forceinline__ float box_distance_f(const MaskK& m, float rx, float ry, float rz) {
+// float, its constants converted once on the host: per-thread conversions of FP64 kernel parameters
+// cost more than the estimate): it decides which points are so far from the surface that tanh(d/delta)
+// is +-1 in the field precision (exactly in FP64 beyond 19.1 delta), where d chi/dtheta vanishes and
+// chi is 0 (outside) or 1 (inside), and the FP64 distance and tanh need not be evaluated.
+struct BoxF {
+  float R[9], x0[3], c[3], hb[3];
+  float far, tol;              // see box_far; a bound of the estimate's error (64 roundings of the largest offset)
+  float h[kMaxLevel + 1];
+};
+inline BoxF box_constants(const MaskK& m, const PhysK& ph, double far) {
+  BoxF b;
+  for (int k = 0; k < 9; ++k) b.R[k] = (float)m.p[k];
+  for (int a = 0; a < 3; ++a) {
+    b.x0[a] = (float)m.p[9 + a];
+    b.c[a] = (float)m.p[12 + a];
+    b.hb[a] = (float)m.p[15 + a];
+  }
+  b.far = (float)far;
+  double E = 0.0;
+  for (int a = 0; a < 3; ++a)
+    E += ph.nroot[a] * ph.root_len + fabs(m.p[9 + a]) + fabs(m.p[12 + a]) + fabs(m.p[15 + a]);
+  b.tol = (float)(64.0 * 6e-8 * E);
+  for (int J = 0; J <= kMaxLevel; ++J) b.h[J] = (float)ph.h[J];
+  return b;
+}
+__device__ __forceinline__ float box_distance_f(const BoxF& b, float rx, float ry, float rz) {
   float n2 = 0.f, qmax = -1e30f;
+#pragma unroll
   for (int k = 0; k < 3; ++k) {
-    const float xb = (float)m.p[k] * rx + (float)m.p[3 + k] * ry + (float)m.p[6 + k] * rz;
-    const float q = fabsf(xb - (float)m.p[12 + k]) - (float)m.p[15 + k];
+    const float xb = b.R[k] * rx + b.R[3 + k] * ry + b.R[6 + k] * rz;
+    const float q = fabsf(xb - b.c[k]) - b.hb[k];
     if (q > 0.f) n2 += q * q;
     qmax = fmaxf(qmax, q);
   }
@@ -115,7 +140,7 @@ __device__ __forceinline__ void box_dus(const MaskK& m, double rx, double ry, do
 // (FP64: tanh rounds to +-1 beyond 19.1 delta; FP32 fields: tanhf beyond 9.1 delta, the FP64
 // derivative left out there is below 1e-8 of its value at the surface).
 template <typename T>
-__device__ __forceinline__ double box_far(const MaskK& m) {
+inline double box_far(const MaskK& m) {
   return (sizeof(T) == 8 ? 20.0 : 10.0) * m.p[18];
 }
 
@@ -146,6 +171,34 @@ __device__ __forceinline__ void block_add(double v, double* out) {
   }
 }
 
+// The stage kernels' constants in the field precision, rounded once on the host: an FP64 division or
+// conversion in every thread's prologue occupies the GPU's few FP64 units longer than the rest of a
+// small kernel takes (576 blocks of 17^3: the face halos 183 us before, with a lookup per component
+// and a kernel of their own for same-level faces, 69 us now; the stage kernel 152 and 142 us).
+template <typename T>
+struct AdjC {
+  T a1, a2, a3, c0sq, inv_ceta, inv_csp, cgam, c_lam, c_nu;
+  T ih[kMaxLevel + 1], nu_ih2[kMaxLevel + 1];      // 1 / h_J, nu / (12 h_J^2)
+};
+template <typename T>
+inline AdjC<T> adj_constants(const AdjStageK<T>& a, const PhysK& ph) {
+  AdjC<T> c;
+  c.a1 = T(ph.a1);
+  c.a2 = T(ph.a2);
+  c.a3 = T(ph.a3);
+  c.c0sq = T(ph.c0sq);
+  c.inv_ceta = T(ph.inv_ceta);
+  c.inv_csp = T(ph.inv_csp);
+  c.cgam = T(ph.cgamma);
+  c.c_lam = T(a.c_lam);
+  c.c_nu = T(a.c_nu);
+  for (int J = 0; J <= kMaxLevel; ++J) {
+    c.ih[J] = T(1.0 / ph.h[J]);
+    c.nu_ih2[J] = T(ph.nu / (12.0 * ph.h[J] * ph.h[J]));
+  }
+  return c;
+}
+
 // ---- the adjoint of one RK stage: nu = W^T E^T loc(E W Y)^T kappa ------------------------------------
 // loc^T kappa at a target point q, for the weights at the block's interior sources p (zero
 // outside the interior; h-free first differences Dt_j g(q) = sum_m a_m [g(q - m e_j) - g(q + m e_j)],
@@ -166,15 +219,17 @@ __device__ __forceinline__ void block_add(double v, double* out) {
 // is read (nu': the next RK stage's nu), and the running sum of the stage nus is updated from nu'
 // in the same pass.  The own targets are stored with plain writes; the targets in the face halos
 // (k_adj_halo) go to other blocks' points through E^T afterwards.
-// A block of 33^3 points is split by rows over three CTAs (as the forward stage kernel): the
+// A block of 33^3 points is split by rows over four CTAs: the
 // kappa rows of the CTA next to this one are sources inside the block, loaded like a halo.
 template <typename T, int BS>
 struct AdjCfg {
-  static constexpr int RY = BS <= 17 ? BS : 11;                  // rows (y) per CTA
+  // rows (y) per CTA.  33^3: four CTAs (9, 9, 9, 6) hold their rings in registers; three of 11 rows spilled
+  // (437 blocks, four gradient steps: 38.9 ms with 11 rows, 33.2 with 9, 34.4 with 7)
+  static constexpr int RY = BS <= 17 ? BS : 9;
   static constexpr int NS = (BS + RY - 1) / RY;                  // CTAs per block
   static constexpr int NT = ((BS * RY + 31) / 32) * 32;
   static constexpr int H = RY + 6;
-  static constexpr int W = sizeof(T) == 4 && BS <= 17 ? BS + 32 : BS + 6;   // bank-conflict-free rows (FP32)
+  static constexpr int W = sizeof(T) == 4 ? BS + 32 : BS + 6;    // bank-conflict-free rows (FP32; 33^3: 33.2 -> 32.8 ms)
   static constexpr int PW = H * W;
   static constexpr int NC = 7;                                   // planes: u, v, w, kappa_0..3
   static constexpr int NHC = 6 * (RY + BS);                      // x/y halo values of one component
@@ -187,11 +242,9 @@ struct AdjCfg {
   static_assert(NS == 1 || sizeof(T) == 4, "row-split blocks are FP32 only");
 };
 
-// MOVING: the moving box's parameter sensitivity (kind 2), compiled apart from the static masks'
-// form so that its FP64 pose arithmetic costs the static form no registers.
-template <typename T, int BS, bool MOVING>
+template <typename T, int BS>
 __global__ void __launch_bounds__(AdjCfg<T, BS>::NT, AdjCfg<T, BS>::MINB)
-k_adj_stage(const AdjStageK<T> a, const TopoK tp, const PhysK ph, const MaskK m) {
+k_adj_stage(const AdjStageK<T> a, const TopoK tp, const PhysK ph, const AdjC<T> kc) {
   using L = Lay<T, BS>;
   using C = AdjCfg<T, BS>;
   constexpr int M = L::M;
@@ -217,11 +270,10 @@ k_adj_stage(const AdjStageK<T> a, const TopoK tp, const PhysK ph, const MaskK m)
   for (int i = tid; i < 2 * C::NC * PW; i += NT) buf[i] = T(0);
   __syncthreads();
 
-  const T a1 = T(ph.a1), a2 = T(ph.a2), a3 = T(ph.a3);
-  const T ih = T(1.0 / ph.h[bi.x]);
-  const T nu_ih2 = T(ph.nu / (12.0 * ph.h[bi.x] * ph.h[bi.x]));
-  const T c0sq = T(ph.c0sq), inv_ceta = T(ph.inv_ceta), inv_csp = T(ph.inv_csp), cgam = T(ph.cgamma);
-  const T c_lam = T(a.c_lam), c_nu = T(a.c_nu);
+  const T a1 = kc.a1, a2 = kc.a2, a3 = kc.a3;
+  const T ih = kc.ih[bi.x], nu_ih2 = kc.nu_ih2[bi.x];
+  const T c0sq = kc.c0sq, inv_ceta = kc.inv_ceta, inv_csp = kc.inv_csp, cgam = kc.cgam;
+  const T c_lam = kc.c_lam, c_nu = kc.c_nu;
   const bool act = tid < BS * ny;
   const int x = act ? tid % BS : 0, y = y0 + (act ? tid / BS : 0);
   const size_t bo = (size_t)slot * L::BLK;
@@ -345,9 +397,6 @@ k_adj_stage(const AdjStageK<T> a, const TopoK tp, const PhysK ph, const MaskK m)
   issue_halos(0, buf);
 
   const int ci = (y - y0 + 3) * W + x + 3;
-  constexpr bool moving = MOVING;
-  double dth = 0.0;
-  const double hd = ph.h[bi.x];
   for (int z = 0; z <= M; ++z) {
     T* B = buf + (z & 1) * C::NC * PW;
     if (act) {
@@ -434,33 +483,8 @@ k_adj_stage(const AdjStageK<T> a, const TopoK tp, const PhysK ph, const MaskK m)
         if (a.sum_mode == 1) a.sum[o] = a.nup[o];
         else if (a.sum_mode == 2) a.sum[o] += a.nup[o];
       }
-      const T u = qy[0][3], v = qy[1][3], w = qy[2][3];
-      if constexpr (MOVING) {
-        const double rx = lattice_coord(ph, bi, 0, x, M, hd) - m.p[9];
-        const double ry = lattice_coord(ph, bi, 1, y, M, hd) - m.p[10];
-        const double rz = lattice_coord(ph, bi, 2, z, M, hd) - m.p[11];
-        const double kk[3] = {(double)k0, (double)k1, (double)k2};
-        const float df = box_distance_f(m, (float)rx, (float)ry, (float)rz);
-        const double far = box_far<T>(m);
-        if (df < -far) {
-          // inside, away from the surface: chi = 1 and d chi = 0, only d u_s/dtheta acts
-          double dus[3], gu = 0.0;
-          box_dus(m, rx, ry, rz, dus);
-          for (int i = 0; i < 3; ++i) gu += (double)chiv * kk[i] * ph.inv_ceta * dus[i];
-          dth += gu;
-        } else if (!(df > far)) {
-          const BoxPoint bp = box_point(m, rx, ry, rz);
-          const double uu[3] = {(double)u, (double)v, (double)w};
-          double gc = 0.0, gu = 0.0;
-          for (int i = 0; i < 3; ++i) {
-            gc -= kk[i] * (uu[i] - bp.us[i]) * ph.inv_ceta;     // d/dchi of -chi (u - u_s) / C_eta
-            gu += (double)chiv * kk[i] * ph.inv_ceta * bp.dus[i]; // d/du_s, times d u_s / dtheta
-          }
-          dth += gc * bp.dchi + gu;
-        }                                                       // outside, far: no term
-      } else if (ph.mask && a.gchi) {
-        a.gchi[(size_t)slot * L::FS + pi] -= (k0 * u + k1 * v + k2 * w) * inv_ceta;
-      }
+      if (ph.mask && a.gchi)
+        a.gchi[(size_t)slot * L::FS + pi] -= (k0 * qy[0][3] + k1 * qy[1][3] + k2 * qy[2][3]) * inv_ceta;
     }
 #pragma unroll
     for (int k = 0; k < 7; ++k) {
@@ -470,10 +494,111 @@ k_adj_stage(const AdjStageK<T> a, const TopoK tp, const PhysK ph, const MaskK m)
       for (int f = 0; f < 4; ++f) qk[f][k] = qk[f][k + 1];
     }
   }
-  if (moving) {
-    __syncthreads();
-    block_add_n<AdjCfg<T, BS>::NT>(dth, a.dtheta);
+}
+
+// The moving box's parameter sensitivity of one RK stage: sum over the points of kappa_i times the
+// derivative of -chi (u_i - u_s,i) / C_eta, through chi near the surface and through u_s inside.  It is
+// FP64 arithmetic on a few points: blocks outside are left at once, and the points of a block that have
+// a term are collected in shared memory so that full warps evaluate them (an FP64 instruction takes the
+// same time for one active lane as for 32).  A block's points go to several CTAs: the blocks around the
+// surface hold nearly all of the work, and a CTA has the FP64 units of one SM only.
+template <int BS>
+struct BodyCfg {
+  static constexpr int P = BS == 33 ? 16 : (BS == 17 ? 2 : 1);      // CTAs per block
+  static constexpr int N = (BS * BS * BS + P - 1) / P;              // points of one
+};
+template <typename T, int BS>
+__global__ void __launch_bounds__(kNA) k_adj_body(const AdjStageK<T> a, const int32_t* blist, const int4* binfo,
+                                                  const PhysK ph, const MaskK m, const BoxF bf, const AdjC<T> kc) {
+  using L = Lay<T, BS>;
+  constexpr int M = L::M;
+  const int rank = blockIdx.x / BodyCfg<BS>::P;
+  const int i0 = (int)(blockIdx.x % BodyCfg<BS>::P) * BodyCfg<BS>::N;
+  const int i1 = i0 + BodyCfg<BS>::N < BS * BS * BS ? i0 + BodyCfg<BS>::N : BS * BS * BS;
+  __shared__ unsigned list[2 * kNA];
+  __shared__ int s_count;
+  const int4 bi = binfo[rank];
+  const float hf = bf.h[bi.x];
+  {
+    // the distance is 1-Lipschitz: its value at the block's centre less the half diagonal bounds it
+    const int g[3] = {bi.y, bi.z, bi.w};
+    bool seam = false;
+    float r[3];
+#pragma unroll
+    for (int k = 0; k < 3; ++k) {
+      seam |= (long long)g[k] + 1 >= ((long long)ph.nroot[k] << bi.x);   // holds points taken as x = 0
+      r[k] = ((float)g[k] * M + 0.5f * M) * hf - bf.x0[k];
+    }
+    if (!seam && box_distance_f(bf, r[0], r[1], r[2]) - 0.8661f * M * hf > bf.far + bf.tol) return;
   }
+  const int tid = threadIdx.x, lane = tid & 31;
+  const size_t bo = (size_t)blist[rank] * L::BLK;
+  const size_t co = (size_t)blist[rank] * L::FS;
+  const double hd = ph.h[bi.x];
+  double dth = 0.0;
+  // entry: point index, bit 31: deep inside (chi = 1 and d chi = 0: only d u_s/dtheta acts)
+  auto term = [&](unsigned e) {
+    const int i = (int)(e & 0x7fffffffu), x = i % BS, y = (i / BS) % BS, z = i / (BS * BS);
+    const size_t pi = (size_t)L::idx(x, y, z);
+    const double rx = lattice_coord(ph, bi, 0, x, M, hd) - m.p[9];
+    const double ry = lattice_coord(ph, bi, 1, y, M, hd) - m.p[10];
+    const double rz = lattice_coord(ph, bi, 2, z, M, hd) - m.p[11];
+    double kk[3];
+#pragma unroll
+    for (int f = 0; f < 3; ++f) {
+      const size_t o = bo + (size_t)f * L::FS + pi;
+      T k = kc.c_lam * a.lam[o];
+      if (a.nup) k += kc.c_nu * a.nup[o];
+      kk[f] = (double)k;
+    }
+    const double ci = (double)a.chi[co + pi] * ph.inv_ceta;
+    if (e & 0x80000000u) {
+      double dus[3];
+      box_dus(m, rx, ry, rz, dus);
+      dth += ci * (kk[0] * dus[0] + kk[1] * dus[1] + kk[2] * dus[2]);
+    } else {
+      const BoxPoint bp = box_point(m, rx, ry, rz);
+      double gc = 0.0, gu = 0.0;
+#pragma unroll
+      for (int f = 0; f < 3; ++f) {
+        gc += kk[f] * ((double)a.Y[bo + (size_t)f * L::FS + pi] - bp.us[f]);
+        gu += kk[f] * bp.dus[f];
+      }
+      dth += ci * gu - ph.inv_ceta * gc * bp.dchi;
+    }
+  };
+  if (tid == 0) s_count = 0;
+  __syncthreads();
+  for (int base = i0; base < i1; base += kNA) {
+    const int i = base + tid;
+    bool has = false;
+    unsigned e = (unsigned)i;
+    if (i < i1) {
+      const int x = i % BS, y = (i / BS) % BS, z = i / (BS * BS);
+      const float df = box_distance_f(bf, (float)lattice_index(ph, bi, 0, x, M) * hf - bf.x0[0],
+                                      (float)lattice_index(ph, bi, 1, y, M) * hf - bf.x0[1],
+                                      (float)lattice_index(ph, bi, 2, z, M) * hf - bf.x0[2]);
+      has = !(df > bf.far);
+      if (df < -bf.far) e |= 0x80000000u;
+    }
+    const unsigned vote = __ballot_sync(0xffffffffu, has);
+    int at = 0;
+    if (lane == 0 && vote) at = atomicAdd(&s_count, __popc(vote));
+    at = __shfl_sync(0xffffffffu, at, 0);
+    if (has) list[at + __popc(vote & ((1u << lane) - 1))] = e;
+    __syncthreads();
+    const int n = s_count;                          // below 2 kNA: at most kNA - 1 were left over
+    __syncthreads();
+    if (n >= kNA) {
+      if (tid == 0) s_count = n - kNA;
+      term(list[n - kNA + tid]);
+      __syncthreads();
+    }
+  }
+  const int n = s_count;
+  if (tid < n) term(list[tid]);
+  __syncthreads();
+  block_add_n<kNA>(dth, a.dtheta);
 }
 
 // The targets of loc^T in block `rank`'s face halos (3 layers beyond each face): only sources
@@ -482,8 +607,8 @@ k_adj_stage(const AdjStageK<T> a, const TopoK tp, const PhysK ph, const MaskK m)
 //             + nu/(12 h^2) sum_{k=l..2} d2_k kappa_i(q -+ k e_n)                      (i < 3)
 //   nu_p(q) = -1/h sum_{m=l..3} (+-a_m) kappa_n(q -+ m e_n)
 // (n the normal axis, the sign that of the face), added through E^T to the point q was read from.
-// One CTA per (block, face); faces toward a same-level neighbour are left to that neighbour,
-// which gathers them (k_adj_samelevel).  Across a finer face q goes to the child's coinciding
+// One CTA per (block, face), a thread per tangential point.  Across a same-level face q is the
+// neighbour's point at distance l inside the shared face; across a finer face q goes to the child's coinciding
 // point (the forward's decimation); fine wins' copies
 // between leaves are W's part (k_adj_fw_T).  Across a coarser face, q is held by a leaf if it lies
 // on one's lattice (its point gets the value), else it was predicted by the tensor DD-4 from the
@@ -541,127 +666,69 @@ __device__ __forceinline__ void face_targets(const AdjStageK<T>& a, const size_t
   }
 }
 
-// E^T across same-level faces in gather form: block A adds to its own points the face-halo
-// targets of its same-level face neighbours that the forward read from A (the neighbour N's
-// halo point at distance l beyond the shared face is A's point at distance l inside it), each
-// computed from N's sources next to the face as k_adj_halo computes a halo target.  One CTA per
-// block walks its six faces in turn (a point near an edge takes one face's value at a time), so
-// the additions need no atomics; a thread per tangential point of a face, all four components.
-// It runs after k_adj_stage and before k_adj_halo's atomics.
-template <int BS>
-struct SameCfg {
-  static constexpr int NT = BS * BS <= 1024 ? ((BS * BS + 31) / 32) * 32 : 384;
-};
-
-template <typename T, int BS>
-__global__ void __launch_bounds__(SameCfg<BS>::NT)
-k_adj_samelevel(const AdjStageK<T> a, const TopoK tp, const PhysK ph, int* err) {
-  using L = Lay<T, BS>;
-  constexpr int M = L::M, NT = SameCfg<BS>::NT;
-  __shared__ int types[6], slots[6];
-  const int rank = blockIdx.x;
-  if (threadIdx.x < 6) {
-    const int d = kFaceBox[threadIdx.x];
-    const int* nbh = tp.nbh + (size_t)rank * kNbhStride;
-    types[threadIdx.x] = nbh[kNbhType + d] & 15;
-    slots[threadIdx.x] = nbh[8 * d];
-  }
-  __syncthreads();
-  const size_t bo = (size_t)tp.blist[rank] * L::BLK;
-  const int4 bi = tp.binfo[rank];
-  const T ih = T(1.0 / ph.h[bi.x]);
-  const T nu_ih2 = T(ph.nu / (12.0 * ph.h[bi.x] * ph.h[bi.x]));
-  const T c0sq = T(ph.c0sq);
-  const T am[3] = {T(ph.a1), T(ph.a2), T(ph.a3)};
-  const T c_lam = T(a.c_lam), c_nu = T(a.c_nu);
-  for (int F = 0; F < 6; ++F) {
-    if (types[F] != kTypeLeaf) continue;                        // uniform over the CTA
-    if (slots[F] < 0) {
-      if (threadIdx.x == 0) atomicOr(err, 8);
-      continue;
-    }
-    const int ax = F >> 1, side = F & 1;
-    const int o1 = ax == 0 ? 1 : 0, o2 = 3 - ax - o1;
-    const size_t nb = (size_t)slots[F] * L::BLK;
-    // the shared face is the neighbour's opposite face: its sources at distance k inside it sit
-    // at neighbour coordinate k (this block's upper face) or M - k (its lower face), and its
-    // halo stencils take the sign of that face
-    const T sg = side ? T(-1) : T(1);
-    for (int uv = threadIdx.x; uv < BS * BS; uv += NT) {
-      int p[3] = {0, 0, 0};
-      p[o1] = uv % BS;
-      p[o2] = uv / BS;
-      size_t po[3];
-#pragma unroll
-      for (int k = 0; k < 3; ++k) {
-        p[ax] = side ? k : M - k;
-        po[k] = nb + L::idx(p[0], p[1], p[2]);
-      }
-      T de[4][3];
-      face_targets<T, BS>(a, po, ax, sg, ih, nu_ih2, c0sq, am, c_lam, c_nu, de);
-#pragma unroll
-      for (int l = 1; l <= 3; ++l) {
-        p[ax] = side ? M - l : l;
-        const size_t o = bo + L::idx(p[0], p[1], p[2]);
-#pragma unroll
-        for (int f = 0; f < 4; ++f) a.nu[o + (size_t)f * L::FS] += de[f][l - 1];
-      }
-    }
-    __syncthreads();
-  }
-}
-
 template <typename T, int BS>
 struct HaloCfg {
   static constexpr int M = BS - 1;
+  static constexpr int NT = BS * BS <= 1024 ? ((BS * BS + 31) / 32) * 32 : 384;   // a thread per tangential point
   static constexpr int NTG = M / 2 + 3;               // even fine tangential coordinates -2 .. M + 2
   static constexpr int NPATCH = 5 * NTG * NTG;        // normal: 5 even fine coordinates beyond the face
   // shared memory of a coarse face: the predicted halo targets h [f][l][t2][t1], then after the
-  // transposed prediction along t1, t2 and the normal a [f][l][t2][c1], b [f][l][c2][c1] (in h's
-  // place) and the patch [f][n][c2][c1] (in a's place)
+  // transposed prediction along t1 and t2 a [f][l][t2][c1] and b [f][l][c2][c1] (in h's place)
   static constexpr int NH3 = 3 * BS * BS, NA = 3 * BS * NTG, NB = 3 * NTG * NTG;
   static constexpr int U0 = 4 * (NH3 > NB ? NH3 : NB);
-  static constexpr int U1 = 4 * (NA > NPATCH ? NA : NPATCH);
+  static constexpr int U1 = 4 * NA;
   static constexpr size_t bytes = (size_t)(U0 + U1) * sizeof(T);
 };
 
 template <typename T, int BS>
-__global__ void __launch_bounds__(kNA) k_adj_halo(const AdjStageK<T> a, const TopoK tp, const PhysK ph, int* err) {
+__global__ void __launch_bounds__(HaloCfg<T, BS>::NT) k_adj_halo(const AdjStageK<T> a, const TopoK tp, const AdjC<T> kc, int* err) {
   using L = Lay<T, BS>;
   using H = HaloCfg<T, BS>;
-  constexpr int M = L::M, NTG = H::NTG, NP = H::NPATCH;
+  constexpr int M = L::M, NTG = H::NTG, NP = H::NPATCH, NT = H::NT;
   __shared__ int nbh[kNbhStride];
   extern __shared__ __align__(16) unsigned char hsm[];
   T* hv = reinterpret_cast<T*>(hsm);                  // h, later b
-  T* acc = hv + H::U0;                                // a, later the patch
+  T* pa = hv + H::U0;                                 // a
   const int rank = blockIdx.x / 6, F = blockIdx.x % 6;
   const int ax = F >> 1, side = F & 1;
   const int d = kFaceBox[F];
-  // a same-level neighbour gathers these targets itself (k_adj_samelevel): its CTA reads the
-  // face's type word only
-  if ((tp.nbh[(size_t)rank * kNbhStride + kNbhType + d] & 15) == kTypeLeaf) return;
-  for (int i = threadIdx.x; i < kNbhStride; i += kNA) nbh[i] = tp.nbh[(size_t)rank * kNbhStride + i];
-  __syncthreads();
-  const int ty = nbh[kNbhType + d] & 15;
+  const int* row = tp.nbh + (size_t)rank * kNbhStride;
+  const int ty = row[kNbhType + d] & 15;
+  int mate = -1;                                      // the leaf beyond a same-level face
+  if (ty == kTypeLeaf) {
+    mate = row[8 * d];
+    if (mate < 0) {
+      if (threadIdx.x == 0) atomicOr(err, 8);
+      return;
+    }
+  } else {
+    for (int i = threadIdx.x; i < kNbhStride; i += NT) nbh[i] = row[i];
+    __syncthreads();
+  }
   const bool coarse = ty != kTypeLeaf && ty != kTypeRefined;
   if (coarse) {
-    for (int i = threadIdx.x; i < 4 * H::NH3; i += kNA) hv[i] = T(0);
+    for (int i = threadIdx.x; i < 4 * H::NH3; i += NT) hv[i] = T(0);
     __syncthreads();
   }
   const size_t bo = (size_t)tp.blist[rank] * L::BLK;
   const int4 bi = tp.binfo[rank];
-  const T ih = T(1.0 / ph.h[bi.x]);
-  const T nu_ih2 = T(ph.nu / (12.0 * ph.h[bi.x] * ph.h[bi.x]));
-  const T c0sq = T(ph.c0sq);
-  const T am[3] = {T(ph.a1), T(ph.a2), T(ph.a3)};
-  const T c_lam = T(a.c_lam), c_nu = T(a.c_nu);
+  const T ih = kc.ih[bi.x], nu_ih2 = kc.nu_ih2[bi.x], c0sq = kc.c0sq;
+  const T am[3] = {kc.a1, kc.a2, kc.a3};
+  const T c_lam = kc.c_lam, c_nu = kc.c_nu;
   // threads run along the tangential axis with the smaller memory stride (x for y and z faces)
   const int o1 = ax == 0 ? 1 : 0, o2 = 3 - ax - o1;
   const T sg = side ? T(1) : T(-1);
   const T wd[4] = {T(-1) / T(16), T(9) / T(16), T(9) / T(16), T(-1) / T(16)};
-  // E^T of one halo target q of component f with value de
-  auto scatter = [&](const int (&q)[3], int f, int l, T de) {
-    if (!coarse) {
+  // E^T of the halo target q at layer l, its four components' values de[.][l - 1]: the place it was read
+  // from is looked up once
+  auto scatter = [&](const int (&q)[3], int l, const T (&de)[4][3]) {
+    long long o = -1;                                 // component 0's element, if a leaf holds q
+    if (ty == kTypeLeaf) {
+      // the neighbour's point at distance l inside the shared face
+      int lc[3] = {q[0], q[1], q[2]};
+      lc[ax] = side ? l : M - l;
+      o = (long long)mate * L::BLK + L::idx(lc[0], lc[1], lc[2]);
+    } else if (!coarse) {
       // a finer face: the child's coinciding point (the forward's decimation)
       int c = (side ? 0 : 1) << ax;
       const int b1 = q[o1] > M / 2, b2 = q[o2] > M / 2;
@@ -675,17 +742,10 @@ __global__ void __launch_bounds__(kNA) k_adj_halo(const AdjStageK<T> a, const To
         atomicOr(err, 8);
         return;
       }
-      if (de != T(0)) atomicAdd(&a.nu[(size_t)s * L::BLK + (size_t)f * L::FS + L::idx(lc[0], lc[1], lc[2])], de);
-      return;
-    }
-    if (de == T(0)) return;
-    if (ty != kTypeCoarser || q[o1] == 0 || q[o1] == M || q[o2] == 0 || q[o2] == M) {
+      o = (long long)s * L::BLK + L::idx(lc[0], lc[1], lc[2]);
+    } else if (ty != kTypeCoarser || q[o1] == 0 || q[o1] == M || q[o2] == 0 || q[o2] == M) {
       // on the face's boundary lines a leaf of this level or finer may hold q
-      const long long o = direct_offset<T, BS>(nbh, q[0], q[1], q[2], f);
-      if (o >= 0) {
-        atomicAdd(&a.nu[o], de);
-        return;
-      }
+      o = direct_offset<T, BS>(nbh, q[0], q[1], q[2], 0);
     } else if (!((q[0] | q[1] | q[2]) & 1)) {
       // strictly inside the face's box only the coarser leaf holds q, on its lattice here
       const int oct = nbh[kNbhType + d] >> 4;
@@ -700,16 +760,21 @@ __global__ void __launch_bounds__(kNA) k_adj_halo(const AdjStageK<T> a, const To
         atomicOr(err, 8);
         return;
       }
-      atomicAdd(&a.nu[(size_t)s * L::BLK + (size_t)f * L::FS + L::idx(lc[0], lc[1], lc[2])], de);
-      return;
+      o = (long long)s * L::BLK + L::idx(lc[0], lc[1], lc[2]);
     }
-    // a predicted ghost: kept for the transposed prediction below (each target has one thread)
-    hv[((f * 3 + l - 1) * BS + q[o2]) * BS + q[o1]] = de;
+    if (o >= 0) {
+#pragma unroll
+      for (int f = 0; f < 4; ++f) atomicAdd(&a.nu[(size_t)o + (size_t)f * L::FS], de[f][l - 1]);
+    } else {
+      // a predicted ghost: kept for the transposed prediction below (each target has one thread)
+#pragma unroll
+      for (int f = 0; f < 4; ++f) hv[((f * 3 + l - 1) * BS + q[o2]) * BS + q[o1]] = de[f][l - 1];
+    }
   };
   // a thread per tangential point, all four components: the three halo layers from the three
   // sources next to the face, p_k at normal distance k = 0, 1, 2 inside it (q at layer l reads
   // p_k with weight a_{l+k}, and its second difference d2_{l+k} for l + k <= 2)
-  for (int uv = threadIdx.x; uv < BS * BS; uv += kNA) {
+  for (int uv = threadIdx.x; uv < BS * BS; uv += NT) {
     int q[3] = {0, 0, 0};
     q[o1] = uv % BS;
     q[o2] = uv / BS;
@@ -725,8 +790,7 @@ __global__ void __launch_bounds__(kNA) k_adj_halo(const AdjStageK<T> a, const To
 #pragma unroll
     for (int l = 1; l <= 3; ++l) {
       q[ax] = side ? M + l : -l;
-#pragma unroll
-      for (int f = 0; f < 4; ++f) scatter(q, f, l, de[f][l - 1]);
+      scatter(q, l, de);
     }
   }
   if (!coarse) return;
@@ -744,53 +808,48 @@ __global__ void __launch_bounds__(kNA) k_adj_halo(const AdjStageK<T> a, const To
     }
     return v;
   };
-  T* pa = acc;
-  for (int i = threadIdx.x; i < 4 * H::NA; i += kNA) {        // along t1: a[f][l][t2][c1]
+  for (int i = threadIdx.x; i < 4 * H::NA; i += NT) {        // along t1: a[f][l][t2][c1]
     const int c1 = i % NTG, r = i / NTG;                      // r = (f * 3 + l) * BS + t2
     pa[i] = gather_line(hv + (size_t)r * BS, 1, 2 * c1 - 2, 0, M);
   }
   __syncthreads();
   T* pb = hv;
-  for (int i = threadIdx.x; i < 4 * H::NB; i += kNA) {        // along t2: b[f][l][c2][c1]
+  for (int i = threadIdx.x; i < 4 * H::NB; i += NT) {        // along t2: b[f][l][c2][c1]
     const int c1 = i % NTG, c2 = (i / NTG) % NTG, fl = i / (NTG * NTG);
     pb[i] = gather_line(pa + (size_t)fl * BS * NTG + c1, NTG, 2 * c2 - 2, 0, M);
   }
   __syncthreads();
   const int nbase = side ? M - 2 : -6;
-  for (int i = threadIdx.x; i < 4 * NP; i += kNA) {           // across the face: patch[f][n][c2][c1]
-    const int c = i % (NTG * NTG), n = (i / (NTG * NTG)) % 5, f = i / NP;
-    // layer l sits at fine normal coordinate side ? M + l : -l, i.e. index l - 1 of b's rows at
-    // coordinate (side ? M + 1 : -1) + (side ? 1 : -1) (l - 1)
-    const int pn = nbase + 2 * n;
-    T v = T(0);
-#pragma unroll
-    for (int l = 1; l <= 3; ++l) {
-      const int qn = side ? M + l : -l;
-      const int off = pn - qn;
-      T w = T(0);
-      if (off == 0) w = T(1);
-      else if (qn & 1) w = off == -3 ? wd[0] : (off == -1 ? wd[1] : (off == 1 ? wd[2] : (off == 3 ? wd[3] : T(0))));
-      if (w != T(0)) v += w * pb[((size_t)(f * 3 + l - 1) * NTG * NTG) + c];
-    }
-    acc[i] = v;
-  }
-  __syncthreads();
-  // each patch point to the leaf holding it (the prediction's sources are held directly)
-  for (int i = threadIdx.x; i < 4 * NP; i += kNA) {
-    const T v = acc[i];
-    if (v == T(0)) continue;
-    const int f = i / NP, r = i % NP;
-    const int kn = r / (NTG * NTG), k2 = (r / NTG) % NTG, k1 = r % NTG;
+  // across the face, a thread per patch point (n, c2, c1): its four components, and the leaf holding it
+  // (the prediction's sources are held directly)
+  for (int i = threadIdx.x; i < NP; i += NT) {
+    const int kn = i / (NTG * NTG), c21 = i % (NTG * NTG), k2 = c21 / NTG, k1 = c21 % NTG;
     int c[3];
     c[ax] = nbase + 2 * kn;
     c[o2] = 2 * k2 - 2;
     c[o1] = 2 * k1 - 2;
-    const long long o = direct_offset<T, BS>(nbh, c[0], c[1], c[2], f);
+    T v[4] = {T(0), T(0), T(0), T(0)};
+    // layer l sits at fine normal coordinate side ? M + l : -l, i.e. index l - 1 of b's rows
+#pragma unroll
+    for (int l = 1; l <= 3; ++l) {
+      const int qn = side ? M + l : -l;
+      const int off = c[ax] - qn;
+      T w = T(0);
+      if (off == 0) w = T(1);
+      else if (qn & 1) w = off == -3 ? wd[0] : (off == -1 ? wd[1] : (off == 1 ? wd[2] : (off == 3 ? wd[3] : T(0))));
+      if (w != T(0)) {
+#pragma unroll
+        for (int f = 0; f < 4; ++f) v[f] += w * pb[(size_t)(f * 3 + l - 1) * NTG * NTG + c21];
+      }
+    }
+    const long long o = direct_offset<T, BS>(nbh, c[0], c[1], c[2], 0);
     if (o < 0) {
-      atomicOr(err, 8);
+      if (v[0] != T(0) || v[1] != T(0) || v[2] != T(0) || v[3] != T(0)) atomicOr(err, 8);
       continue;
     }
-    atomicAdd(&a.nu[o], v);
+#pragma unroll
+    for (int f = 0; f < 4; ++f)
+      if (v[f] != T(0)) atomicAdd(&a.nu[(size_t)o + (size_t)f * L::FS], v[f]);
   }
 }
 
@@ -849,12 +908,45 @@ __global__ void __launch_bounds__(kNA) k_adj_fw_T(T* r, const int2* tasks, const
   }
 }
 
-// out = x + y + z over the blocks of the list (whole block strides).
+// Block-wise streams over the registers run kParts CTAs per block and whole 16-byte words, several in
+// flight per thread: with one CTA per block and a word at a time they left half of the HBM rate unused
+// (x + y + z of 440 blocks of 33^3: 327 us).
+constexpr int kParts = 4;
+template <typename T>
+struct alignas(16) Word { T v[16 / sizeof(T)]; };
+
+// out = x + y + z over the blocks of the list (whole block strides); out may be x.
 template <typename T, int BS>
 __global__ void __launch_bounds__(kNA) k_adj_sum3(T* out, const T* x, const T* y, const T* z, const int32_t* blist) {
   using L = Lay<T, BS>;
-  const size_t base = (size_t)blist[blockIdx.x] * L::BLK;
-  for (int i = threadIdx.x; i < L::BLK; i += kNA) out[base + i] = x[base + i] + y[base + i] + z[base + i];
+  constexpr int V = 16 / (int)sizeof(T), NW = L::BLK / V, STEP = kNA * kParts, U = 4;
+  static_assert(L::BLK % V == 0, "a block is a whole number of 16-byte words");
+  const size_t base = (size_t)blist[blockIdx.x / kParts] * L::BLK;
+  const Word<T>* xw = reinterpret_cast<const Word<T>*>(x + base);
+  const Word<T>* yw = reinterpret_cast<const Word<T>*>(y + base);
+  const Word<T>* zw = reinterpret_cast<const Word<T>*>(z + base);
+  Word<T>* ow = reinterpret_cast<Word<T>*>(out + base);
+  for (int i0 = (blockIdx.x % kParts) * kNA + threadIdx.x; i0 < NW; i0 += U * STEP) {
+    Word<T> a[U], b[U], c[U];
+#pragma unroll
+    for (int u = 0; u < U; ++u) {
+      const int i = i0 + u * STEP;
+      if (i < NW) {
+        a[u] = xw[i];
+        b[u] = yw[i];
+        c[u] = zw[i];
+      }
+    }
+#pragma unroll
+    for (int u = 0; u < U; ++u) {
+      const int i = i0 + u * STEP;
+      if (i < NW) {
+#pragma unroll
+        for (int k = 0; k < V; ++k) a[u].v[k] = a[u].v[k] + b[u].v[k] + c[u].v[k];
+        ow[i] = a[u];
+      }
+    }
+  }
 }
 
 // Direct terms of (1/N) [F_x(U) + w_E E(U)] (Sec. 2.2, half-open points, weight h^3): into lam
@@ -864,7 +956,8 @@ __global__ void __launch_bounds__(kNA) k_adj_sum3(T* out, const T* x, const T* y
 template <typename T, int BS>
 __global__ void __launch_bounds__(kNA) k_adj_objective(const T* U, const T* chi, T* lam, T* gchi,
                                                        const int32_t* blist, const int4* binfo, const PhysK ph,
-                                                       double wN, double wE, const MaskK m, double* dtheta) {
+                                                       double wN, double wE, const MaskK m, const BoxF bf,
+                                                       double* dtheta) {
   using L = Lay<T, BS>;
   constexpr int M = L::M;
   const int slot = blist[blockIdx.x];
@@ -887,13 +980,12 @@ __global__ void __launch_bounds__(kNA) k_adj_objective(const T* U, const T* chi,
       const double rx = lattice_coord(ph, bi, 0, x, M, h) - m.p[9];
       const double ry = lattice_coord(ph, bi, 1, y, M, h) - m.p[10];
       const double rz = lattice_coord(ph, bi, 2, z, M, h) - m.p[11];
-      const float df = box_distance_f(m, (float)rx, (float)ry, (float)rz);
-      const double far = box_far<T>(m);
-      if (df < -far) {                          // chi = 1, d chi = 0: the u_s term only
+      const float df = box_distance_f(bf, (float)rx, (float)ry, (float)rz);
+      if (df < -bf.far) {                       // chi = 1, d chi = 0: the u_s term only
         double dus[3];
         box_dus(m, rx, ry, rz, dus);
         dth += wN * h3 * ph.inv_ceta * (0.0 - c * dus[0]);
-      } else if (!(df > far)) {
+      } else if (!(df > bf.far)) {
         const BoxPoint bp = box_point(m, rx, ry, rz);
         dth += wN * h3 * ph.inv_ceta * ((u - bp.us[0]) * bp.dchi - c * bp.dus[0]);
       }
@@ -948,12 +1040,22 @@ __global__ void __launch_bounds__(kNA) k_adj_theta(const T* gchi, const int32_t*
 template <typename T, int BS>
 __global__ void __launch_bounds__(kNA) k_adj_gather(const T* r, double* dense, const int32_t* blist) {
   using L = Lay<T, BS>;
-  constexpr int N3 = BS * BS * BS;
-  const size_t own = (size_t)blist[blockIdx.x] * L::BLK;
-  double* d = dense + (size_t)blockIdx.x * 4 * N3;
-  for (int t = threadIdx.x; t < 4 * N3; t += kNA) {
-    const int f = t / N3, r3 = t % N3;
-    d[t] = (double)r[own + (size_t)f * L::FS + L::idx(r3 % BS, (r3 / BS) % BS, r3 / (BS * BS))];
+  constexpr int N3 = BS * BS * BS, PAD = L::PP - BS * BS;
+  const int f = blockIdx.x % 4, rank = blockIdx.x / 4;                  // a CTA per block and component
+  const T* s = r + (size_t)blist[rank] * L::BLK + (size_t)f * L::FS;
+  double* d = dense + ((size_t)rank * 4 + f) * N3;
+  for (int t = threadIdx.x; t < N3; t += 8 * kNA) {
+    T v[8];
+#pragma unroll
+    for (int u = 0; u < 8; ++u) {
+      const int j = t + u * kNA;
+      if (j < N3) v[u] = s[j + j / (BS * BS) * PAD];
+    }
+#pragma unroll
+    for (int u = 0; u < 8; ++u) {
+      const int j = t + u * kNA;
+      if (j < N3) d[j] = (double)v[u];
+    }
   }
 }
 
@@ -962,12 +1064,22 @@ __global__ void __launch_bounds__(kNA) k_adj_gather(const T* r, double* dense, c
 template <typename T, int BS>
 __global__ void __launch_bounds__(kNA) k_adj_put(const double* dense, T* r, const int32_t* blist) {
   using L = Lay<T, BS>;
-  constexpr int N3 = BS * BS * BS;
-  const size_t own = (size_t)blist[blockIdx.x] * L::BLK;
-  const double* d = dense + (size_t)blockIdx.x * 4 * N3;
-  for (int t = threadIdx.x; t < 4 * N3; t += kNA) {
-    const int f = t / N3, r3 = t % N3;
-    r[own + (size_t)f * L::FS + L::idx(r3 % BS, (r3 / BS) % BS, r3 / (BS * BS))] = T(d[t]);
+  constexpr int N3 = BS * BS * BS, PAD = L::PP - BS * BS;
+  const int f = blockIdx.x % 4, rank = blockIdx.x / 4;
+  T* o = r + (size_t)blist[rank] * L::BLK + (size_t)f * L::FS;
+  const double* d = dense + ((size_t)rank * 4 + f) * N3;
+  for (int t = threadIdx.x; t < N3; t += 8 * kNA) {
+    double v[8];
+#pragma unroll
+    for (int u = 0; u < 8; ++u) {
+      const int j = t + u * kNA;
+      if (j < N3) v[u] = d[j];
+    }
+#pragma unroll
+    for (int u = 0; u < 8; ++u) {
+      const int j = t + u * kNA;
+      if (j < N3) o[j + j / (BS * BS) * PAD] = T(v[u]);
+    }
   }
 }
 
@@ -986,18 +1098,17 @@ inline unsigned fw_ctas(int64_t max_tasks) {
 template <typename T, int BS>
 void stage(const AdjStageK<T>& a, const TopoK& t, const PhysK& ph, const MaskK& m, const FwTasks& fw, int* err,
            cudaStream_t st) {
-  static std::atomic<unsigned long long> opted{0}, opted_m{0};
-  if (m.kind == 2) {
-    smem_opt_in_stage(k_adj_stage<T, BS, true>, AdjCfg<T, BS>::bytes, opted_m);
-    k_adj_stage<T, BS, true><<<g1(t.n * AdjCfg<T, BS>::NS), AdjCfg<T, BS>::NT, AdjCfg<T, BS>::bytes, st>>>(a, t, ph, m);
-  } else {
-    smem_opt_in_stage(k_adj_stage<T, BS, false>, AdjCfg<T, BS>::bytes, opted);
-    k_adj_stage<T, BS, false><<<g1(t.n * AdjCfg<T, BS>::NS), AdjCfg<T, BS>::NT, AdjCfg<T, BS>::bytes, st>>>(a, t, ph, m);
-  }
-  k_adj_samelevel<T, BS><<<g1(t.n), SameCfg<BS>::NT, 0, st>>>(a, t, ph, err);
+  static std::atomic<unsigned long long> opted{0};
+  const AdjC<T> kc = adj_constants<T>(a, ph);
+  AdjStageK<T> as = a;
+  if (m.kind == 2) as.gchi = nullptr;               // the body's kernel forms its sensitivity itself
+  smem_opt_in_stage(k_adj_stage<T, BS>, AdjCfg<T, BS>::bytes, opted);
+  k_adj_stage<T, BS><<<g1(t.n * AdjCfg<T, BS>::NS), AdjCfg<T, BS>::NT, AdjCfg<T, BS>::bytes, st>>>(as, t, ph, kc);
+  if (m.kind == 2)
+    k_adj_body<T, BS><<<g1(t.n * BodyCfg<BS>::P), kNA, 0, st>>>(a, t.blist, t.binfo, ph, m, box_constants(m, ph, box_far<T>(m)), kc);
   static std::atomic<unsigned long long> opted_h{0};
   smem_opt_in_stage(k_adj_halo<T, BS>, HaloCfg<T, BS>::bytes, opted_h);
-  k_adj_halo<T, BS><<<g1(6 * t.n), kNA, HaloCfg<T, BS>::bytes, st>>>(a, t, ph, err);
+  k_adj_halo<T, BS><<<g1(6 * t.n), HaloCfg<T, BS>::NT, HaloCfg<T, BS>::bytes, st>>>(a, t, kc, err);
   k_adj_fw_T<T, BS><<<fw_ctas(fw.max_tasks), kNA, 0, st>>>(a.nu, fw.tasks, fw.ntasks, t.nbh, t.blist);
 }
 
@@ -1008,13 +1119,14 @@ void fw_T(T* r, const FwTasks& fw, const int32_t* blist, const int32_t* nbh, cud
 
 template <typename T, int BS>
 void sum3(T* out, const T* x, const T* y, const T* z, const int32_t* blist, int64_t n, cudaStream_t st) {
-  k_adj_sum3<T, BS><<<g1(n), kNA, 0, st>>>(out, x, y, z, blist);
+  k_adj_sum3<T, BS><<<g1(n * kParts), kNA, 0, st>>>(out, x, y, z, blist);
 }
 
 template <typename T, int BS>
 void objective(const T* U, const T* chi, T* lam, T* gchi, const int32_t* blist, const int4* binfo,
                int64_t n, const PhysK& ph, double wN, double wE, const MaskK& m, double* dtheta, cudaStream_t st) {
-  k_adj_objective<T, BS><<<g1(n), kNA, 0, st>>>(U, chi, lam, gchi, blist, binfo, ph, wN, wE, m, dtheta);
+  k_adj_objective<T, BS><<<g1(n), kNA, 0, st>>>(U, chi, lam, gchi, blist, binfo, ph, wN, wE, m,
+                                             box_constants(m, ph, box_far<T>(m)), dtheta);
 }
 
 template <typename T, int BS>
@@ -1025,12 +1137,12 @@ void theta(const T* gchi, const int32_t* blist, const int4* binfo, int64_t n, co
 
 template <typename T, int BS>
 void gather(const T* r, double* dense, const int32_t* blist, int64_t n, cudaStream_t st) {
-  k_adj_gather<T, BS><<<g1(n), kNA, 0, st>>>(r, dense, blist);
+  k_adj_gather<T, BS><<<g1(4 * n), kNA, 0, st>>>(r, dense, blist);
 }
 
 template <typename T, int BS>
 void put(const double* dense, T* r, const int32_t* blist, int64_t n, cudaStream_t st) {
-  k_adj_put<T, BS><<<g1(n), kNA, 0, st>>>(dense, r, blist);
+  k_adj_put<T, BS><<<g1(4 * n), kNA, 0, st>>>(dense, r, blist);
 }
 
 }  // namespace adj

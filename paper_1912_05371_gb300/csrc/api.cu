@@ -467,6 +467,7 @@ void plate_pose(acm_forest* f, double t) {
   m.p[33] = -dw * sp;
   m.p[34] = dw * cp;
   m.p[35] = 0.0;
+  m.p[36] = 1.0 / q[9];            // 1 / delta
 }
 
 // Mask on every block, or only on the blocks whose slots are in `fresh` (new blocks).
@@ -1241,7 +1242,7 @@ acm_status adjoint_sweep(acm_forest* f, int nsteps, double dt, int c, double wE,
     a.gchi = GCHI;
     a.dtheta = TH;
     acm::launch_adj_stage<T>(Bs, a, tk_topo, f->phk, cur_mask(), fwt, f->d_err, f->st);
-    f->launches += 5;
+    f->launches += plate ? 5 : 4;
     return cudaGetLastError() == cudaSuccess ? ACM_OK : fail(f, ACM_ECUDA, "adjoint kernel launch failed");
   };
   auto objective = [&](const T* Us, double tn) {
