@@ -501,7 +501,8 @@ k_adj_stage(const AdjStageK<T> a, const TopoK tp, const PhysK ph, const AdjC<T> 
 // FP64 arithmetic on a few points: blocks outside are left at once, and the points of a block that have
 // a term are collected in shared memory so that full warps evaluate them (an FP64 instruction takes the
 // same time for one active lane as for 32).  A block's points go to several CTAs: the blocks around the
-// surface hold nearly all of the work, and a CTA has the FP64 units of one SM only.
+// surface hold nearly all of the work, and a CTA has the FP64 units of one SM only (blocks of 33^3 around a
+// plate: 913 us per stage with a CTA per block, 194 with 16).
 template <int BS>
 struct BodyCfg {
   static constexpr int P = BS == 33 ? 16 : (BS == 17 ? 2 : 1);      // CTAs per block
