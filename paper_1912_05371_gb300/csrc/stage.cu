@@ -40,6 +40,7 @@
 #include <type_traits>
 
 #include "stage_common.cuh"
+#include "stage_parts.hpp"
 
 namespace acm {
 
@@ -66,6 +67,7 @@ struct Cfg {
   static constexpr int MINB = sizeof(T) == 4 ? (NT <= 160 ? 4 : 2) : 1;   // CTAs per SM
   static_assert(NS == 1 || sizeof(T) == 4, "row-split blocks are FP32 only");
   static_assert(PW < 0x8000, "plane buffer offsets must fit 15 bits");
+  static_assert(parts_are_sound(BS), "the upper halo planes arrive before they are read, for every part");
 };
 
 // Shared planes.  FP32: a point's (u, v, w, p) is one float4.  FP64: (u, v) and (w, p) in two
@@ -632,7 +634,8 @@ __device__ __forceinline__ void stage_block(const StagePtrs<T>& a, const StageCo
     if ((tid & 31) == 0) mbar_arrive(&full[sl]);
   };
   // The planes beyond the upper z face, needed from iteration M - 2 on (each thread its own pencil's),
-  // requested far enough ahead that nobody waits for them.
+  // requested far enough ahead that nobody waits for them; which iteration commits their group is
+  // upper_in_prologue / upper_in_loop's rule (stage_parts.hpp).
   auto load_upper = [&]() {
     const T* p;
     int ls, fcs;
@@ -651,7 +654,7 @@ __device__ __forceinline__ void stage_block(const StagePtrs<T>& a, const StageCo
   };
   int ds = 0, dp = 0;                     // slot and phase of the iteration
   if (work) {
-    if (SPLIT && act && z0 >= M - 2) load_upper();
+    if (SPLIT && act && upper_in_prologue(z0, M)) load_upper();
     issue_halos(z0);
     if (!SPLIT || z0 + 1 < z1) issue_halos(z0 + 1);
     else cp_async_commit();
@@ -673,7 +676,7 @@ __device__ __forceinline__ void stage_block(const StagePtrs<T>& a, const StageCo
       const T* sg = stg + (size_t)ds * nst * SP;
       ds = ds == kND - 1 ? 0 : ds + 1;
       dp ^= ds == 0;
-      if (z == z0 + 1 && act && (!SPLIT || (z0 < M - 2 && z1 > M - 2))) load_upper();
+      if (act && upper_in_loop(z, z0, z1, M)) load_upper();
       if (z + 2 < z1) issue_halos(z + 2);
       else cp_async_commit();
       if (z + 1 < z1) {
@@ -751,7 +754,8 @@ k_stage(const StageK<T> a, const TopoK tp, const PhysK ph, int* err, int nz) {
   constexpr int NS = Cfg<T, BS>::NS;
   if (!SPLIT) nz = 1;
   const int rank = blockIdx.x / (NS * nz), q = blockIdx.x % (NS * nz), zp = q / NS;
-  stage_block<T, BS, STAGE, PM, false, SPLIT>(a.p, a.kc, tp, ph, err, rank, q % NS, zp * BS / nz, (zp + 1) * BS / nz);
+  stage_block<T, BS, STAGE, PM, false, SPLIT>(a.p, a.kc, tp, ph, err, rank, q % NS, part_begin(zp, nz, BS),
+                                              part_begin(zp + 1, nz, BS));
 }
 
 // Persistent form over several independent instances: the CTAs walk the work list of
@@ -804,17 +808,7 @@ __global__ void k_rk_coefs(const unsigned long long* maxbits, RkK p, double* rk)
 template <typename T, int BS>
 int z_parts(int64_t n) {
   using C = Cfg<T, BS>;
-  const int64_t slots = (int64_t)C::MINB * sm_count(), start = sizeof(T) == 4 ? 5 : 1;
-  int best = 1;
-  int64_t cost = -1;
-  for (int nz = 1; nz <= BS / 2; ++nz) {
-    const int64_t c = (n * C::NS * nz + slots - 1) / slots * (start + (BS + nz - 1) / nz);
-    if (cost < 0 || c < cost) {
-      cost = c;
-      best = nz;
-    }
-  }
-  return best;
+  return z_parts_rule(n, C::NS, BS, (int64_t)C::MINB * sm_count(), sizeof(T) == 4 ? 5 : 1);
 }
 
 template <typename T, int BS, int STAGE, bool PM, bool SPLIT>
