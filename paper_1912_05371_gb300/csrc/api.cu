@@ -89,6 +89,7 @@ struct acm_forest {
   int tune_fw_ctas = 8;            // fine-wins kernel: CTAs per SM walking the task list
   int tune_slab_ctas = 3;          // coarse-face slab kernel: CTAs per SM walking the task list
   float tune_stage_ms = 0.f;       // the autotuner's time of one stage launch (FP32)
+  int stage_parts = 0;             // parts of a block along z (0: the stage kernel's own rule)
 
   // host side of the current topology (the neighbourhood tables are built on the device from
   // the block list; the host leaf map is brought up to date only when a host query needs it)
@@ -568,6 +569,7 @@ acm_status rk4(acm_forest* f, double dt, double* dt_used, T* const* save = nullp
     acm::StageK<T> a{};
     a.p = stage_ptrs<T>(f, s, save);
     a.point_major = save == nullptr;
+    a.parts = f->stage_parts;
     a.c_acc = s == 1 ? dt / 6.0 : dt / 3.0;
     a.c_out = s == 1 || s == 2 ? dt / 2.0 : (s == 3 ? dt : dt / 6.0);
     a.body = f->moving ? &f->mask : nullptr;
@@ -628,6 +630,7 @@ acm_status enqueue_rk4_device_dt(acm_forest* f, double dt, int64_t side_by_side 
     a.p = stage_ptrs<T>(f, s);
     a.point_major = 1;
     a.side_by_side = side_by_side;
+    a.parts = f->stage_parts;
     a.p.coefp = f->d_rk + 2;
     if (s == 4) CK(cudaMemsetAsync(f->d_maxbits, 0, 8 * sizeof(unsigned long long), f->st));
     acm::launch_stage<T>(s, f->gp.Bs, a, t, f->phk, f->d_err, f->st);
@@ -1968,6 +1971,18 @@ acm_status acm_set_stage_variant(acm_forest* f, int variant) {
   if (variant != ACM_STAGE_PAIR && variant != ACM_STAGE_POINT && variant != ACM_STAGE_POINT_TMA &&
       variant != ACM_STAGE_POINT_ROWS)
     return fail(f, ACM_EINVAL, "unknown stage kernel");
+  return ACM_OK;
+}
+
+// Not part of the C ABI (the header does not declare it): the parts of a block along z in this forest's
+// stage launches, 1 .. Bs / 2, or 0 for the kernel's own rule, which follows the block count and the
+// chip.  The tests visit every count with it.  Drops a captured graph (it holds the old launches).
+acm_status acm_internal_stage_parts(acm_forest* f, int parts) {
+  if (!f) return ACM_EINVAL;
+  if (parts < 0 || parts > f->gp.Bs / 2) return fail(f, ACM_EINVAL, "parts along z out of range");
+  f->stage_parts = parts;
+  if (f->gexec) { cudaGraphExecDestroy(f->gexec); f->gexec = nullptr; }
+  if (f->graph) { cudaGraphDestroy(f->graph); f->graph = nullptr; }
   return ACM_OK;
 }
 

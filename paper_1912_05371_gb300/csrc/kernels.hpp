@@ -108,6 +108,7 @@ struct StageK {
   StagePtrs<T> p;
   double c_acc, c_out;      // stage coefficients (see stage.cu)
   int64_t side_by_side;     // blocks that run at the same time on other streams included (0: this grid's)
+  int parts;                // parts of a block along z, 1 .. Bs / 2 (0: chosen by the rule in stage.cu)
   int point_major;          // layout of the stage states and the accumulator (see stage.cu At)
   const MaskK* body;        // host: a moving body's pose (its u_s enters the penalization), or null
   StageConst<T> kc;         // the constants in the field precision (filled by launch_stage)

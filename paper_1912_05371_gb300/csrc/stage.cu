@@ -821,7 +821,7 @@ void launch_parts(const StageK<T>& s, const TopoK& t, const PhysK& p, int* err, 
 }
 template <typename T, int BS, int STAGE, bool PM>
 void launch_one(const StageK<T>& s, const TopoK& t, const PhysK& p, int* err, cudaStream_t st) {
-  const int nz = PM ? z_parts<T, BS>(std::max(t.n, s.side_by_side)) : 1;
+  const int nz = !PM ? 1 : (s.parts > 0 ? s.parts : z_parts<T, BS>(std::max(t.n, s.side_by_side)));
   if constexpr (PM) {
     if (nz > 1) {
       launch_parts<T, BS, STAGE, PM, true>(s, t, p, err, nz, st);
