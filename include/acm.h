@@ -290,7 +290,9 @@ acm_status acm_get_tuning(const acm_forest* f, acm_tuning* out);
  * at every ckpt-th step and recomputes each segment with its states stored; ckpt < 0 is binomial
  * checkpointing with -ckpt snapshots (the fewest recomputed steps for that memory).  Every
  * schedule takes the same steps in the same arithmetic, so the result does not depend on it
- * (up to the order of floating-point atomic sums).  ws: caller device buffer of at least
+ * (up to the order of floating-point atomic sums).  On a grid of one level the gradient with
+ * respect to the state has no such sum and is repeatable to the last bit; on graded grids, and
+ * for the mask parameters, the order of the additions is open.  ws: caller device buffer of at least
  * acm_adjoint_bytes(f, nsteps, ckpt) bytes (ACM_ENOMEM if smaller): nine registers and the
  * snapshots in the forest's precision, with ckpt > 0 also the four RK stage states of each of a
  * segment's min(ckpt, nsteps) - 1 recomputed steps (a recomputed step keeps them for its

@@ -10,8 +10,8 @@ namespace acm {
 namespace adj {
 
 template <typename T, int BS>
-void stage(const AdjStageK<T>& a, const TopoK& t, const PhysK& ph, const MaskK& m, const FwTasks& fw, int* err,
-           cudaStream_t st);
+void stage(const AdjStageK<T>& a, const TopoK& t, const PhysK& ph, const MaskK& m, const FwTasks& fw, bool one_level,
+           int* err, cudaStream_t st);
 template <typename T, int BS>
 void fw_T(T* r, const FwTasks& fw, const int32_t* blist, const int32_t* nbh, cudaStream_t st);
 template <typename T, int BS>
@@ -43,9 +43,9 @@ void put(const double* dense, T* r, const int32_t* blist, int64_t n, cudaStream_
 
 template <typename T>
 void launch_adj_stage(int Bs, const AdjStageK<T>& a, const TopoK& t, const PhysK& ph, const MaskK& m,
-                      const FwTasks& fw, int* err, cudaStream_t st) {
+                      const FwTasks& fw, bool one_level, int* err, cudaStream_t st) {
   if (t.n <= 0) return;
-  ACM_ADJ_BS(Bs, stage, a, t, ph, m, fw, err, st);
+  ACM_ADJ_BS(Bs, stage, a, t, ph, m, fw, one_level, err, st);
 }
 
 template <typename T>
@@ -91,7 +91,7 @@ void launch_adj_put(int Bs, const double* dense, T* r, const int32_t* blist, int
 
 #define ACM_ADJ_INST(T)                                                                                        \
   template void launch_adj_stage<T>(int, const AdjStageK<T>&, const TopoK&, const PhysK&, const MaskK&,         \
-                                    const FwTasks&, int*, cudaStream_t);                                      \
+                                    const FwTasks&, bool, int*, cudaStream_t);                                \
   template void launch_adj_fw_T<T>(int, T*, const FwTasks&, const int32_t*, const int32_t*, int64_t, cudaStream_t); \
   template void launch_adj_sum3<T>(int, T*, const T*, const T*, const T*, const int32_t*, int64_t, cudaStream_t); \
   template void launch_adj_objective<T>(int, const T*, const T*, T*, T*, const int32_t*, const int4*, int64_t,  \

@@ -15,7 +15,8 @@
 //                    of the stage nus and the mask sensitivity fused in;
 //   k_adj_body       the moving body's parameter sensitivity (a moving body only);
 //   k_adj_halo       loc^T at the face-halo points and E^T: added to the points they were read from
-//                    (the finest leaf holding the point, or its DD-4 prediction's even points);
+//                    (the finest leaf holding the point, or its DD-4 prediction's even points), or on
+//                    grids of one level k_adj_samelevel, which gathers them in a fixed order;
 //   k_adj_fw_T       W^T: a boundary point held by a finer leaf passes its value to that leaf's
 //                    point and is cleared.
 // The objective's direct terms and the reduction of the mask sensitivity onto the sphere's centre
@@ -667,6 +668,79 @@ __device__ __forceinline__ void face_targets(const AdjStageK<T>& a, const size_t
   }
 }
 
+// The same on grids of one level, in gather form: block A adds to its own points the face-halo targets
+// of its neighbours that the forward read from A (the neighbour's halo point at distance l beyond the
+// shared face is A's point at distance l inside it), each computed from the neighbour's sources next to
+// the face.  The additions need no atomics and their order is fixed, x, y, z: a point near an edge takes
+// one axis's value at a time, the two faces of an axis reach different points, and the two CTAs of a
+// block own the points of its lower and its upper half in z.  So gradients with respect to the state are
+// repeatable to the last bit where every neighbour is of the block's own level.  (On graded grids finer
+// and coarser faces reach the same points, so their order is open in any case.)  Bound by latency: each
+// thread has its 12 values of nu, 15 or 27 source values and then 12 stores in flight at once.  Gradient of
+// four steps, us with k_adj_halo's atomics and with this kernel: FP32, 64 blocks of 17^3 1657 and 1602, 512
+// blocks 4440 and 4309, 4096 blocks 27800 and 27200; 64 blocks of 33^3 5736 and 5385; 4096 blocks of 9^3
+// 6860 and 6290; FP64, 64 blocks of 17^3 11500 with either.
+template <int BS>
+struct SameCfg {
+  static constexpr int ZH = BS / 2 + 1;                                 // planes of the lower half
+  static constexpr int NT = BS <= 17 ? ((2 * BS * ZH + 31) / 32) * 32 : 384;
+};
+
+template <typename T, int BS>
+__global__ void __launch_bounds__(SameCfg<BS>::NT)
+k_adj_samelevel(const AdjStageK<T> a, const TopoK tp, const AdjC<T> kc, int* err) {
+  using L = Lay<T, BS>;
+  constexpr int M = L::M, ZH = SameCfg<BS>::ZH;
+  static_assert(ZH > 3 && M - 3 >= ZH, "a half holds the three layers inside its z face, and no others");
+  const int rank = blockIdx.x >> 1, half = blockIdx.x & 1;
+  const int z0 = half ? ZH : 0, nz = half ? BS - ZH : ZH;
+  const int32_t* fr = tp.faces + (size_t)rank * kFaceStride;
+  const size_t bo = (size_t)tp.blist[rank] * L::BLK;
+  const int4 bi = tp.binfo[rank];
+  const T am[3] = {kc.a1, kc.a2, kc.a3};
+#pragma unroll
+  for (int ax = 0; ax < 3; ++ax) {
+    // threads run along x, for x faces along y
+    const int rows = ax == 2 ? BS : nz, nf = BS * rows, ne = ax == 2 ? nf : 2 * nf;
+    for (int e = threadIdx.x; e < ne; e += SameCfg<BS>::NT) {
+      const int side = ax == 2 ? half : e / nf, r = ax == 2 ? e : e % nf, F = 2 * ax + side;
+      const int mate = fr[6 + 4 * F];
+      if (fr[F] != kTypeLeaf || mate < 0) {
+        if (r == 0) atomicOr(err, 8);
+        continue;
+      }
+      int p[3] = {0, 0, 0};
+      p[ax == 0 ? 1 : 0] = r % BS;
+      p[ax == 2 ? 1 : 2] = (ax == 2 ? 0 : z0) + r / BS;
+      // the shared face is the neighbour's opposite face: its sources at distance k inside it sit at
+      // neighbour coordinate k (this block's upper face) or M - k (its lower face), and its halo
+      // stencils take the sign of that face
+      size_t po[3];
+#pragma unroll
+      for (int k = 0; k < 3; ++k) {
+        p[ax] = side ? k : M - k;
+        po[k] = (size_t)mate * L::BLK + L::idx(p[0], p[1], p[2]);
+      }
+      size_t o[3];
+      T v[4][3], de[4][3];
+#pragma unroll
+      for (int l = 1; l <= 3; ++l) {
+        p[ax] = side ? M - l : l;
+        o[l - 1] = bo + L::idx(p[0], p[1], p[2]);
+#pragma unroll
+        for (int f = 0; f < 4; ++f) v[f][l - 1] = a.nu[o[l - 1] + (size_t)f * L::FS];
+      }
+      face_targets<T, BS>(a, po, ax, side ? T(-1) : T(1), kc.ih[bi.x], kc.nu_ih2[bi.x], kc.c0sq, am, kc.c_lam, kc.c_nu,
+                          de);
+#pragma unroll
+      for (int l = 0; l < 3; ++l)
+#pragma unroll
+        for (int f = 0; f < 4; ++f) a.nu[o[l] + (size_t)f * L::FS] = v[f][l] + de[f][l];
+    }
+    __syncthreads();
+  }
+}
+
 template <typename T, int BS>
 struct HaloCfg {
   static constexpr int M = BS - 1;
@@ -1097,8 +1171,8 @@ inline unsigned fw_ctas(int64_t max_tasks) {
 }
 
 template <typename T, int BS>
-void stage(const AdjStageK<T>& a, const TopoK& t, const PhysK& ph, const MaskK& m, const FwTasks& fw, int* err,
-           cudaStream_t st) {
+void stage(const AdjStageK<T>& a, const TopoK& t, const PhysK& ph, const MaskK& m, const FwTasks& fw, bool one_level,
+           int* err, cudaStream_t st) {
   static std::atomic<unsigned long long> opted{0};
   const AdjC<T> kc = adj_constants<T>(a, ph);
   AdjStageK<T> as = a;
@@ -1107,9 +1181,13 @@ void stage(const AdjStageK<T>& a, const TopoK& t, const PhysK& ph, const MaskK& 
   k_adj_stage<T, BS><<<g1(t.n * AdjCfg<T, BS>::NS), AdjCfg<T, BS>::NT, AdjCfg<T, BS>::bytes, st>>>(as, t, ph, kc);
   if (m.kind == 2)
     k_adj_body<T, BS><<<g1(t.n * BodyCfg<BS>::P), kNA, 0, st>>>(a, t.blist, t.binfo, ph, m, box_constants(m, ph, box_far<T>(m)), kc);
-  static std::atomic<unsigned long long> opted_h{0};
-  smem_opt_in_stage(k_adj_halo<T, BS>, HaloCfg<T, BS>::bytes, opted_h);
-  k_adj_halo<T, BS><<<g1(6 * t.n), HaloCfg<T, BS>::NT, HaloCfg<T, BS>::bytes, st>>>(a, t, kc, err);
+  if (one_level) {
+    k_adj_samelevel<T, BS><<<g1(2 * t.n), SameCfg<BS>::NT, 0, st>>>(a, t, kc, err);
+  } else {
+    static std::atomic<unsigned long long> opted_h{0};
+    smem_opt_in_stage(k_adj_halo<T, BS>, HaloCfg<T, BS>::bytes, opted_h);
+    k_adj_halo<T, BS><<<g1(6 * t.n), HaloCfg<T, BS>::NT, HaloCfg<T, BS>::bytes, st>>>(a, t, kc, err);
+  }
   k_adj_fw_T<T, BS><<<fw_ctas(fw.max_tasks), kNA, 0, st>>>(a.nu, fw.tasks, fw.ntasks, t.nbh, t.blist);
 }
 
@@ -1153,8 +1231,8 @@ void put(const double* dense, T* r, const int32_t* blist, int64_t n, cudaStream_
 #define ACM_ADJ_INSTANTIATE(T, BS)                                                                                 \
   namespace acm {                                                                                                  \
   namespace adj {                                                                                                  \
-  template void stage<T, BS>(const AdjStageK<T>&, const TopoK&, const PhysK&, const MaskK&, const FwTasks&, int*,  \
-                             cudaStream_t);                                                                        \
+  template void stage<T, BS>(const AdjStageK<T>&, const TopoK&, const PhysK&, const MaskK&, const FwTasks&, bool,  \
+                             int*, cudaStream_t);                                                                  \
   template void fw_T<T, BS>(T*, const FwTasks&, const int32_t*, const int32_t*, cudaStream_t);                       \
   template void sum3<T, BS>(T*, const T*, const T*, const T*, const int32_t*, int64_t, cudaStream_t);                \
   template void objective<T, BS>(const T*, const T*, T*, T*, const int32_t*, const int4*, int64_t,                   \

@@ -1252,7 +1252,7 @@ acm_status adjoint_sweep(acm_forest* f, int nsteps, double dt, int c, double wE,
     a.sum_mode = sum_mode;
     a.gchi = GCHI;
     a.dtheta = TH;
-    acm::launch_adj_stage<T>(Bs, a, tk_topo, f->phk, cur_mask(), fwt, f->d_err, f->st);
+    acm::launch_adj_stage<T>(Bs, a, tk_topo, f->phk, cur_mask(), fwt, f->one_level, f->d_err, f->st);
     f->launches += (plate ? 4 : 3) + (f->one_level ? 0 : 1);
     return cudaGetLastError() == cudaSuccess ? ACM_OK : fail(f, ACM_ECUDA, "adjoint kernel launch failed");
   };

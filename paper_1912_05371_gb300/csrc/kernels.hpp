@@ -276,10 +276,11 @@ struct FwTasks {
   const int32_t* ntasks;
   int64_t max_tasks;
 };
-// err |= 8 if a ghost point's source is missing.
+// err |= 8 if a ghost point's source is missing.  one_level: every block has the same level (the halo
+// targets are then gathered in a fixed order, without atomics).
 template <typename T>
 void launch_adj_stage(int Bs, const AdjStageK<T>& a, const TopoK& t, const PhysK& ph, const MaskK& m,
-                      const FwTasks& fw, int* err, cudaStream_t st);
+                      const FwTasks& fw, bool one_level, int* err, cudaStream_t st);
 // W^T applied to register r in place (n: blocks of the grid).
 template <typename T>
 void launch_adj_fw_T(int Bs, T* r, const FwTasks& fw, const int32_t* blist, const int32_t* nbh, int64_t n,
