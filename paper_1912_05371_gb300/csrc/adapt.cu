@@ -629,10 +629,11 @@ k_details_big(const T* reg, const T* chi, const int32_t* blist, const int32_t* r
 }
 
 // ---- (5) max norms (Sec. 2.3 u_max, Sec. 3.4 normalisation) ------------------------------------
-template <typename T, int BS>
-__global__ void __launch_bounds__(kNT) k_maxnorm(const T* reg, const int32_t* blist, unsigned long long* out, int parts) {
+// P: CTAs per block.
+template <typename T, int BS, int P>
+__global__ void __launch_bounds__(kNT) k_maxnorm(const T* reg, const int32_t* blist, unsigned long long* out) {
   using L = Lay<T, BS>;
-  const int slot = blist[blockIdx.x / parts];
+  const int slot = blist[blockIdx.x / P];
   const T* b = reg + (size_t)slot * L::BLK;
   // arithmetic in the field precision (an FP32 field gives an FP32 norm, stored as double);
   // m[4] holds the squared magnitude, its root is taken once at the end.  The maxima propagate
@@ -640,7 +641,7 @@ __global__ void __launch_bounds__(kNT) k_maxnorm(const T* reg, const int32_t* bl
   // reaches the host as a non-finite norm.
   T m[5] = {T(0), T(0), T(0), T(0), T(0)};
   constexpr int N = BS * BS * BS, U = 4;
-  for (int base = (blockIdx.x % parts) * kNT * U + threadIdx.x; base < N; base += parts * kNT * U) {
+  for (int base = (blockIdx.x % P) * kNT * U + threadIdx.x; base < N; base += P * kNT * U) {
     T v[U][4];
 #pragma unroll
     for (int k = 0; k < U; ++k) {
@@ -1773,9 +1774,24 @@ void launch_details(int Bs, const T* reg, const T* chi, const int32_t* blist, co
 template <typename T>
 void launch_maxnorm(int Bs, const T* reg, const int32_t* blist, int64_t n, unsigned long long* out, cudaStream_t st) {
   if (n <= 0) return;
-  // a grid of fewer blocks than the chip holds CTAs (eight per SM) splits each over four
-  const int parts = n < 8 * sm_count() ? 4 : 1;
-  ACM_BS_DISPATCH(Bs, k_maxnorm, <<<grid1(n * parts), kNT, 0, st>>>(reg, blist, out, parts));
+  // Blocks over four CTAs each on grids that leave the chip idle: 17^3 with fewer blocks than SMs, 33^3 (five
+  // times the passes per CTA) with fewer than the chip holds CTAs, eight per SM.  More CTAs cost more atomic
+  // maxima on the same five words, and a 9^3 block is one pass of a CTA, so the line lies there.  A
+  // diagnostics call, us, with one CTA per block and with four: FP64 17^3 8 blocks 59.5 and 55.6, 302 blocks
+  // 75.2 and 96.2, 1009 blocks 176 and 220; FP32 17^3 64 blocks 51.2 and 48.7, 1009 blocks 126 and 134; 33^3
+  // 64 blocks 130 and 119, 631 blocks 440 and 428; 9^3 FP32 302 blocks 48.3 and 57.5.
+  const bool split = n < (Bs == 33 ? 8 : (Bs == 17 ? 1 : 0)) * sm_count();
+  if (Bs == 33) {
+    if constexpr (sizeof(T) == 4) {
+      if (split) k_maxnorm<T, 33, 4><<<grid1(n * 4), kNT, 0, st>>>(reg, blist, out);
+      else k_maxnorm<T, 33, 1><<<grid1(n), kNT, 0, st>>>(reg, blist, out);
+    }
+  } else if (Bs == 17) {
+    if (split) k_maxnorm<T, 17, 4><<<grid1(n * 4), kNT, 0, st>>>(reg, blist, out);
+    else k_maxnorm<T, 17, 1><<<grid1(n), kNT, 0, st>>>(reg, blist, out);
+  } else {
+    k_maxnorm<T, 9, 1><<<grid1(n), kNT, 0, st>>>(reg, blist, out);
+  }
 }
 template <typename T, int BS>
 void launch_refine_bs(const T* src, T* dst, const int32_t* tasks, int64_t n, const int32_t* blist,
