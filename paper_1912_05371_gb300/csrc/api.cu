@@ -51,7 +51,6 @@ struct acm_forest {
   int32_t* d_nbh = nullptr;
   int4* d_binfo = nullptr;
   int32_t* d_blist = nullptr;
-  int32_t* d_slabidx = nullptr;
   int32_t* d_faces = nullptr;
   int2* d_fw = nullptr;
   int4* d_slabt = nullptr;
@@ -222,7 +221,6 @@ size_t carve(acm_forest* f, const acm_grid_params* g, char* base) {
   int32_t* nbh = c.take<int32_t>(nb * acm::kNbhStride * 4);
   int4* binfo = c.take<int4>(nb * 16);
   int32_t* blist = c.take<int32_t>(nb * 4);
-  int32_t* slabidx = c.take<int32_t>(nb * 8 * 4);
   int32_t* faces = c.take<int32_t>(nb * acm::kFaceStride * 4);
   int2* fw = c.take<int2>(nb * 26 * 8);
   int4* slabt = c.take<int4>(nb * 6 * 16);
@@ -247,8 +245,7 @@ size_t carve(acm_forest* f, const acm_grid_params* g, char* base) {
   double* rk = c.take<double>(32 * 8);
   if (f) {
     f->U = U; f->ACC = ACC; f->YA = YA; f->YB = YB; f->CHI = CHI; f->DENSE = DENSE; f->SLAB = SLAB;
-    f->d_nbh = nbh; f->d_binfo = binfo; f->d_blist = blist; f->d_slabidx = slabidx;
-    f->d_faces = faces;
+    f->d_nbh = nbh; f->d_binfo = binfo; f->d_blist = blist; f->d_faces = faces;
     f->d_fw = fw; f->d_slabt = slabt; f->d_reft = reft; f->d_crst = crst; f->d_ranks = ranks;
     f->d_norms = norms; f->d_maxbits = maxbits; f->d_ind = ind; f->d_chir = chir; f->d_diag = diag;
     f->d_err = errf;
@@ -264,7 +261,6 @@ acm::TopoK topo(const acm_forest* f) {
   t.nbh = f->d_nbh;
   t.binfo = f->d_binfo;
   t.blist = f->d_blist;
-  t.slabidx = f->d_slabidx;
   t.faces = f->d_faces;
   t.n = (int64_t)f->order.size();
   return t;
@@ -337,8 +333,8 @@ acm_status upload_topology(acm_forest* f, std::vector<BoxKey>* new_order = nullp
   tk.mask = (unsigned long long)(f->leaf_cap - 1);
   for (int a = 0; a < 3; ++a) tk.nroot[a] = f->gp.nroot[a];
   acm::launch_topology(tk, f->d_ltab, f->d_bslot, f->d_binfo, f->d_blist, n, f->d_nbh, f->d_finer, f->d_fwmask,
-                       f->d_slabmask, f->d_fwoff, f->d_slaboff, f->d_counts, f->d_fw, f->d_slabt, f->d_slabidx,
-                       f->d_faces, f->d_err, f->st);
+                       f->d_slabmask, f->d_fwoff, f->d_slaboff, f->d_counts, f->d_fw, f->d_slabt, f->d_faces,
+                       f->d_err, f->st);
   CKL();
   f->launches += 4;
   f->host_rows_ms += now_ms() - t1;

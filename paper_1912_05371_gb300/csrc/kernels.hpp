@@ -33,12 +33,12 @@ struct TreeK {
 
 // Rebuild the device leaf table (tab, box) from the blocks binfo/blist[0..n) of the current order,
 // then the neighbourhood rows (nbh, rank-indexed), the per-block flag "a neighbour box is
-// refined" (finer), and the fine-wins task list (fw) and coarse-face slab list (slabt, slabidx);
+// refined" (finer), and the fine-wins task list (fw) and coarse-face slab list (slabt);
 // counts[0], counts[1] receive the two list lengths.  fwmask/slabmask/fw_off/slab_off: per-block
 // scratch.  err |= 2 if the grid is not graded, |= 4 if the table overflowed.
 void launch_topology(const TreeK& t, int* tab, int4* box, const int4* binfo, const int32_t* blist, int64_t n,
                      int32_t* nbh, uint8_t* finer, uint32_t* fwmask, uint32_t* slabmask, int32_t* fw_off,
-                     int32_t* slab_off, int32_t* counts, int2* fw, int4* slabt, int32_t* slabidx, int32_t* faces, int* err,
+                     int32_t* slab_off, int32_t* counts, int2* fw, int4* slabt, int32_t* faces, int* err,
                      cudaStream_t st);
 
 // Device topology: pointers into the pool, all indexed by rank (position in block order).
@@ -46,7 +46,6 @@ struct TopoK {
   const int32_t* nbh;       // [n][kNbhStride] neighbourhood tables
   const int4* binfo;        // [n] (J, gx, gy, gz)
   const int32_t* blist;     // [n] slot of each block
-  const int32_t* slabidx;   // [n][8]: coarse-face halo slab per face (-1: none)
   // [n][kFaceStride] what the stage kernels read of a block's faces F = 0 -x, 1 +x, 2 -y, 3 +y, 4 -z,
   // 5 +z, in one line: words 0..5 the neighbour's type (leaf, refined or coarser), words 6 + 4F + j
   // its slot (leaf), the slots of the four children touching the face (refined, j = first + 2 x

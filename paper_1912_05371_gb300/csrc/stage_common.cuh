@@ -76,10 +76,6 @@ __device__ __forceinline__ float d2_first(float2 c, float2 m1, float2 p1, float2
 __device__ __forceinline__ double d2_first(double2 c, double2 m1, double2 p1, double2 m2, double2 p2) {
   return fma(30.0, c.x, fma(-16.0, p1.x + m1.x, p2.x + m2.x));
 }
-// Bulk prefetch of a contiguous range into L2 (address and size multiples of 16 bytes).
-__device__ __forceinline__ void prefetch_l2(const void* p, unsigned bytes) {
-  asm volatile("cp.async.bulk.prefetch.L2.global [%0], %1;\n" ::"l"(p), "r"(bytes) : "memory");
-}
 __device__ __forceinline__ void cp_async_commit() { asm volatile("cp.async.commit_group;\n" ::: "memory"); }
 
 __device__ __forceinline__ unsigned smem_u32(const void* p) { return (unsigned)__cvta_generic_to_shared(p); }
@@ -116,10 +112,6 @@ __device__ __forceinline__ void mbar_wait(unsigned long long* bar, unsigned pari
       " add.u32 n, n, 1;\n setp.lt.u32 p, n, 4194304;\n @p bra W%=;\n red.global.or.b32 [%2], 1;\n"
       "D%=:\n}\n" ::"r"(smem_u32(bar)), "r"(parity), "l"(err)
       : "memory");
-}
-// this thread's earlier cp.async copies arrive on the mbarrier when they have completed
-__device__ __forceinline__ void cp_async_mbar_arrive(unsigned long long* bar) {
-  asm volatile("cp.async.mbarrier.arrive.noinc.shared::cta.b64 [%0];\n" ::"r"(smem_u32(bar)) : "memory");
 }
 template <int N>
 __device__ __forceinline__ void cp_async_wait_group() {

@@ -236,11 +236,10 @@ __global__ void __launch_bounds__(kScanNT) k_scan(const uint32_t* fwmask, const 
 }
 
 // Task lists in block order, then ascending box index / face: fine-wins task (rank, d) per refined
-// neighbour box; slab (rank, face, index) per face covered by a coarser leaf, and the block's
-// slab index per face (-1: none).
+// neighbour box; slab (rank, face, index) per face covered by a coarser leaf, whose index also goes
+// to the block's face record.
 __global__ void __launch_bounds__(256) k_fill(const uint32_t* fwmask, const uint32_t* slabmask, const int32_t* fw_off,
-                                              const int32_t* slab_off, int64_t n, int2* fw, int4* slabt,
-                                              int32_t* slabidx, int32_t* faces) {
+                                              const int32_t* slab_off, int64_t n, int2* fw, int4* slabt, int32_t* faces) {
   const int64_t r = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
   if (r >= n) return;
   const uint32_t m = fwmask[r];
@@ -249,35 +248,29 @@ __global__ void __launch_bounds__(256) k_fill(const uint32_t* fwmask, const uint
     if ((m >> d) & 1u) fw[j++] = make_int2((int)r, d);
   const uint32_t sm = slabmask[r];
   int k = slab_off[r];
-  for (int F = 0; F < 8; ++F) {
-    int idx = -1;
-    if (F < 6 && ((sm >> F) & 1u)) {
-      idx = k++;
+  for (int F = 0; F < 6; ++F)
+    if ((sm >> F) & 1u) {
+      const int idx = k++;
       slabt[idx] = make_int4((int)r, F, idx, 0);
-    }
-    slabidx[r * 8 + F] = idx;
-    if (idx >= 0)
       for (int q = 0; q < 4; ++q) faces[r * kFaceStride + 6 + 4 * F + q] = idx;
-  }
+    }
 }
 
 }  // namespace
 
 void launch_topology(const TreeK& t, int* tab, int4* box, const int4* binfo, const int32_t* blist, int64_t n,
                      int32_t* nbh, uint8_t* finer, uint32_t* fwmask, uint32_t* slabmask, int32_t* fw_off,
-                     int32_t* slab_off, int32_t* counts, int2* fw, int4* slabt, int32_t* slabidx, int32_t* faces,
-                     int* err, cudaStream_t st) {
+                     int32_t* slab_off, int32_t* counts, int2* fw, int4* slabt, int32_t* faces, int* err,
+                     cudaStream_t st) {
   cudaMemsetAsync(tab, 0xff, (size_t)(t.mask + 1) * sizeof(int), st);
   if (n <= 0) {
     cudaMemsetAsync(counts, 0, 2 * sizeof(int32_t), st);
     return;
   }
   k_index<<<(unsigned)((n + 255) / 256), 256, 0, st>>>(t, binfo, blist, n, tab, box, err);
-  k_rows<<<(unsigned)((n * 32 + 255) / 256), 256, 0, st>>>(t, binfo, n, nbh, finer, fwmask, slabmask, faces,
-                                                                  err);
+  k_rows<<<(unsigned)((n * 32 + 255) / 256), 256, 0, st>>>(t, binfo, n, nbh, finer, fwmask, slabmask, faces, err);
   k_scan<<<1, kScanNT, 0, st>>>(fwmask, slabmask, n, fw_off, slab_off, counts);
-  k_fill<<<(unsigned)((n + 255) / 256), 256, 0, st>>>(fwmask, slabmask, fw_off, slab_off, n, fw, slabt, slabidx,
-                                                         faces);
+  k_fill<<<(unsigned)((n + 255) / 256), 256, 0, st>>>(fwmask, slabmask, fw_off, slab_off, n, fw, slabt, faces);
 }
 
 }  // namespace acm
