@@ -67,10 +67,9 @@ typedef enum {
 /* Grid of cubic blocks (Sec. 4.1).  nroot[3] roots of side root_len tile the periodic box
  * [0, nroot*root_len]; a block at level J has side root_len/2^J and spacing
  * h_J = root_len / (2^J (Bs-1)).  Bs is 9, 17 or 33; Bs = 33 takes precision 32 and the CDF 4/0
- * wavelet (ACM_EINVAL otherwise), and its forests have no adjoint (acm_adjoint_* return
- * ACM_EINVAL) and no persistent batched form (acm_rk4_steps_batch falls back to the graph of
- * per-instance launches).  g is the ghost depth reported by
- * acm_sync_ghosts (1..4).  precision is 32 or 64.  fd_scheme: 1 = Tam-Webb optimised first
+ * wavelet (ACM_EINVAL otherwise), and its forests have no persistent batched form
+ * (acm_rk4_steps_batch falls back to the graph of per-instance launches).  g is the ghost depth
+ * reported by acm_sync_ghosts (1..4).  precision is 32 or 64.  fd_scheme: 1 = Tam-Webb optimised first
  * derivative (Sec. 2.3, the paper's choice), 0 = classical (8,-1)/12.  Levels obey
  * 0 <= Jmin <= Jmax <= 18 (Sec. 3.5).  max_blocks (the block pool) is below 2^32 divided by
  * the larger of a block's padded element count and 72 Bs^2 (about 206,000 blocks at Bs = 17,
@@ -235,7 +234,9 @@ acm_status acm_rk4_steps(acm_forest* f, int nsteps, double dt, int use_graph, do
  * second is captured into one CUDA graph and replayed.  It needs forests of one precision and
  * block size with identical physics and grid spacings, and uses forests[0]'s staging buffer
  * (the one acm_read_fields/acm_write_fields use) for its instance table and work list; otherwise
- * the call takes use_graph = 1.  *graph_used receives 0 (plain launches), 1 or 2.  The persistent
+ * the call takes use_graph = 1.  For several forests at a time this call is the fast one: a forest
+ * stepped by itself is laid out as if it had the GPU alone (small grids spread over all of it).
+ * *graph_used receives 0 (plain launches), 1 or 2.  The persistent
  * form computes every block's update bitwise as the other forms do.  Synchronises every stream at
  * the end; t_end (may be NULL) receives n simulated times.  Errors are reported on the forest
  * concerned (forests[0] for capture errors and the persistent stage launches).  No counterpart in
@@ -263,7 +264,7 @@ acm_status acm_autotune(acm_forest* f, int* fw_ctas, int* slab_ctas);
 #define ACM_STAGE_POINT 1
 #define ACM_STAGE_POINT_TMA 2
 #define ACM_STAGE_POINT_ROWS 3
-/* Accepts the names above (they select the same kernel); drops a captured graph.  ACM_EINVAL for
+/* Accepts the names above (they select the same kernel, so nothing changes).  ACM_EINVAL for
  * another value. */
 acm_status acm_set_stage_variant(acm_forest* f, int variant);
 

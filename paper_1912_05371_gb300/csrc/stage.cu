@@ -29,8 +29,9 @@
 // restriction) or, across a face to a coarser neighbour, from the halo slab that the coarse-face
 // kernel predicted for this stage.  No ghost layer is written to HBM.
 //
-// What bounds it: shared-memory wavefronts (58 % of the cycles on large FP32 grids) and the prologue of a
-// CTA (halo table, first planes), then HBM; FP64: the FP64 pipe.  Measured per launch (mean over the four
+// What bounds it: the L1 data pipe's wavefronts (68, 55, 55 and 51 % of the cycles in stages 1 to 4 on 4608
+// FP32 blocks; 60, 48, 48 and 45 % are shared-memory ones), latency at two CTAs per SM and the prologue of
+// a CTA (halo table, first planes), then HBM (1.10 times the algorithmic bytes); FP64: the FP64 pipe.  Measured per launch (mean over the four
 // stages), against one point per thread with a point's components apart and the accumulator kept:
 // 4608 blocks of 17^3 FP32 0.393 ms (0.434 before); 32768 blocks 2.42 (2.79); 64 blocks 0.0192 (0.0297);
 // 33^3 moving plate 1.57 (2.23, its solid-velocity kernel included); FP64 4096 blocks 2.37 (2.63).  Slower
@@ -800,11 +801,13 @@ __global__ void k_rk_coefs(const unsigned long long* maxbits, RkK p, double* rk)
 // planes; the parts are chosen so that the waves of CTAs over the chip cost least: a grid of a few
 // dozen blocks would leave most of the SMs idle with one CTA per block.  n: the blocks that run side by
 // side (instances of a batch on several streams together fill a chip that one of them would not: with
-// each split by its own count a batch of 12 instances took 11.1 ms instead of 9.9).  Measured, ms per launch with
-// one part and with this rule's: 64 blocks of 17^3 FP32 0.0192 and 0.0133, FP64 0.213 and 0.116; FP64
-// 1472 blocks 2.365 and 2.347.  A grid that fills the chip keeps one part, in a form of the kernel
-// whose plane range the compiler knows (the split form spills registers there: 4608 blocks 0.426
-// against 0.393, 32768 blocks 2.63 against 2.42).
+// each split by its own count a batch of 12 instances took 11.1 ms instead of 9.9).  Measured, us per
+// launch with one part and with this rule's: 17^3 FP32 8 blocks 19.0 and 9.4 (six parts), 57 blocks 20.9
+// and 13.1 (five), 64 blocks 19.1 and 13.4 (four); FP64 29 blocks 212 and 57 (five), 64 blocks 210 and 114
+// (two), 512 blocks 827 and 745 (two); 64 blocks of 33^3 65.0 and 54.8 (three), of 9^3 in FP64 53.3 and 33.0
+// (two).  Where it keeps one part, two cost more: 302 blocks of 17^3 FP32 27.8 and 34.2.  A grid that fills
+// the chip keeps one part, in a form of the kernel whose plane range the compiler knows (the split form
+// spills registers there: 4608 blocks 426 against 393 us, 32768 blocks 2630 against 2420).
 template <typename T, int BS>
 int z_parts(int64_t n) {
   using C = Cfg<T, BS>;
